@@ -321,9 +321,17 @@ __device__ __forceinline__ void transpose_sum(float (&v)[NV], int lane) {
 #ifndef EPIKV_TOKEN_OWN_OFFSET
 #define EPIKV_TOKEN_OWN_OFFSET 1  // 0: one-token calls also look the row up through shared memory
 #endif
-template <int LH, int SEG = kLagSeg, bool HALF = false, int KINDS = 0>
+//
+// The stream's tokens [t_lo, t_hi) of the call's n_new are taken: all of them,
+// or (SPLIT) one piece of a long call, cut at chunk boundaries by
+// lag_piece so that few sequences still fill the GPU.  A later piece forms
+// its first chunk's previous range from that chunk's rows (bf16 minima and
+// maxima, the same in any order) and leaves the saved state alone; the first
+// piece, the only one that reads the state, also writes the state that the
+// whole call leaves, from the call's last rows.
+template <int LH, int SEG = kLagSeg, bool HALF = false, int KINDS = 0, bool SPLIT = false>
 __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, const KvDev& kv, int seq,
-                                           int n_new, int layer, int kvk, int nc0) {
+                                           int t_lo, int t_hi, int n_new, int layer, int kvk, int nc0) {
   const int stream = layer * 2 + kvk;  // this stream's column of the per-token partials
   const int tid = HALF ? (int)(threadIdx.x & 127) : (int)threadIdx.x;
   const int nthr = HALF ? 128 : (int)blockDim.x;
@@ -343,7 +351,7 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
   f32x2 na[4], nc[4];
   {
     uint4 pmn = cmn, pmx = cmn;
-    if (active && need_norm) {
+    if (active && need_norm && !(SPLIT && t_lo > 0)) {
       pmn = *reinterpret_cast<const uint4*>(rng + 0 * hd + ch);
       pmx = *reinterpret_cast<const uint4*>(rng + 1 * hd + ch);
       cmn = *reinterpret_cast<const uint4*>(rng + 2 * hd + ch);
@@ -356,19 +364,52 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
   const char* kvbase = kvk ? kv.base[1] : kv.base[0];  // a select: no local copy of the parameter struct
   const char* kvb_ch = kvbase + (int64_t)ch * 2;       // this thread's first channel in a row at offset 0
   __shared__ int64_t soff_s[HALF ? 2 : 1][kLagOffs];
+  int64_t* soff = soff_s[half];
+  const bool whole = !SPLIT || (t_lo == 0 && t_hi == n_new);   // the call's only piece of this stream
+
+  // minimum and maximum of this thread's channels over the call's tokens [a, b), a < b
+  auto range_of = [&](int a, int b, uint4& mn, uint4& mx) {
+    bool first = true;
+    for (int g0 = a; g0 < b; g0 += kLagOffs) {
+      const int gn = min(kLagOffs, b - g0);
+      __syncthreads();
+      for (int t = tid; t < gn; t += nthr) soff[t] = kv_row_offset(kv, layer, seq, nc0 + g0 + t, dm.T);
+      __syncthreads();
+      for (int i = 0; i < gn; i += kLagSeg) {
+        uint4 x[kLagSeg];
+#pragma unroll
+        for (int j = 0; j < kLagSeg; ++j) {   // past the end: the last row again
+          const int64_t off = soff[min(i + j, gn - 1)];
+          x[j] = ld_stream16_if(kvb_ch + off * 2, active && off >= 0);
+        }
+        if (first) mn = mx = x[0];
+        first = false;
+#pragma unroll
+        for (int j = 0; j < kLagSeg; ++j) {
+          mn = q_min(mn, x[j]);
+          mx = q_max(mx, x[j]);
+        }
+      }
+    }
+  };
+
+  if (SPLIT && t_lo > 0 && need_norm) {
+    uint4 pmn, pmx;
+    range_of(t_lo - dm.lag, t_lo, pmn, pmx);
+    prev_affine(pmn, pmx, dm.lag_eps, na, nc);
+  }
   constexpr int NV = 2 * SEG;      // moments of a segment: (sum y, sum y^2) per token
   __shared__ float red_s[HALF ? 2 : 1][2][32][NV];  // [half][segment parity][head][moment]; the host admits H <= 32
   __shared__ float hr_s[HALF ? 2 : 1][2][SEG][32];  // raw variances, same layout
-  int64_t* soff = soff_s[half];
   float (*red)[32][NV] = red_s[half];
   float (*hr)[SEG][32] = hr_s[half];
   float* part = need_norm ? st.lag_part + (size_t)seq * dm.max_new * (2 * dm.L) : nullptr;
   float* rpart = need_raw ? st.raw_part + (size_t)seq * dm.max_new * (2 * dm.L) : nullptr;
-  int r = p0 % dm.lag;                   // position of the next token inside its chunk
+  int r = (p0 + t_lo) % dm.lag;          // position of the next token inside its chunk
   int parity = 0;
 
-  for (int g0 = 0; g0 < n_new; g0 += kLagOffs) {
-    const int gn = min(kLagOffs, n_new - g0);
+  for (int g0 = t_lo; g0 < t_hi; g0 += kLagOffs) {
+    const int gn = min(kLagOffs, t_hi - g0);
     // one-token calls: every thread looks its row up itself (one broadcast
     // load per warp), so no shared table and none of its two barriers.  The
     // SEG == 1 instances run only in the decode-step kernel, whose calls
@@ -504,13 +545,28 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
       r += seg;
       if (r == dm.lag) {  // chunk complete: it becomes the previous chunk
         prev_affine(cmn, cmx, dm.lag_eps, na, nc);
-        if (active && need_norm) {
+        if (active && need_norm && whole) {
           *reinterpret_cast<uint4*>(rng + 0 * hd + ch) = cmn;
           *reinterpret_cast<uint4*>(rng + 1 * hd + ch) = cmx;
         }
         r = 0;
       }
       i += seg;
+    }
+  }
+  if (SPLIT && !whole) {
+    if (t_lo > 0 || !need_norm) return;
+    // the state after the call's last token: its last complete chunk's range
+    // and the running one (all of these rows are the call's, lag_piece)
+    const int tail = (p0 + n_new) % dm.lag, tc = n_new - tail;
+    uint4 pmn, pmx;
+    range_of(tc - dm.lag, tc, pmn, pmx);
+    cmn = pmn;
+    cmx = pmx;
+    if (tail) range_of(tc, n_new, cmn, cmx);
+    if (active) {
+      *reinterpret_cast<uint4*>(rng + 0 * hd + ch) = pmn;
+      *reinterpret_cast<uint4*>(rng + 1 * hd + ch) = pmx;
     }
   }
   if (active && need_norm) {
@@ -527,11 +583,26 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
 #else
 #define EPIKV_LAG_BOUNDS __launch_bounds__(256, EPIKV_LAG_MINB)
 #endif
-template <int LH, int KINDS>
+// Piece z of a call's n_new tokens starting at position p0, in pieces of
+// `piece` tokens (a multiple of lag, at least 4 * lag; 0: one piece): the
+// cuts lie at chunk boundaries, the first piece is two chunks shorter (it
+// reads up to that much at the end of the call for the state), and the rows
+// of the chunk before every cut belong to the call.
+__device__ __forceinline__ int lag_piece_start(int p0, int lag, int piece, int z) {
+  return z == 0 ? 0 : (lag - p0 % lag) % lag + z * piece - 2 * lag;
+}
+// grid.z that covers max_new tokens from any position
+static int lag_pieces(int max_new, int lag, int piece) {
+  return piece ? (max_new + 2 * lag + piece - 1) / piece : 1;
+}
+
+// SPLIT: the instance that takes calls in pieces (the other keeps the
+// registers of one piece).
+template <int LH, int KINDS, bool SPLIT>
 __global__ void EPIKV_LAG_BOUNDS lagkv_partial_kernel(DevState st, Dims dm, KvDev kv,
                                                              const int32_t* __restrict__ seq_ids,
                                                              const int32_t* __restrict__ cu_new,
-                                                             int max_new) {
+                                                             int max_new, int piece) {
   pdl_wait();
   pdl_trigger();
   const int b = blockIdx.y;
@@ -548,7 +619,14 @@ __global__ void EPIKV_LAG_BOUNDS lagkv_partial_kernel(DevState st, Dims dm, KvDe
     if (threadIdx.x == 0) set_error(st.err, EPIKV_DEV_CAPACITY);
     return;
   }
-  lag_stream<LH, kLagSeg, false, KINDS>(st, dm, kv, seq, n_new, layer, kvk, nc0);
+  int t_lo = 0, t_hi = n_new;
+  if (SPLIT) {
+    const int p0 = st.n_seen[seq], z = blockIdx.z;
+    t_lo = lag_piece_start(p0, dm.lag, piece, z);
+    t_hi = min(n_new, lag_piece_start(p0, dm.lag, piece, z + 1));
+    if (t_lo >= n_new && z > 0) return;
+  }
+  lag_stream<LH, kLagSeg, false, KINDS, SPLIT>(st, dm, kv, seq, t_lo, t_hi, n_new, layer, kvk, nc0);
 }
 
 #ifndef EPIKV_FIN_TILE
@@ -999,8 +1077,8 @@ __global__ void __launch_bounds__(kGThreads, EPIKV_TOKEN_MINB) token_kernel(DevS
     const int layer = half ? sidx : sidx >> 1;
     // the new row's slot: this layer's own length under per-layer budgets
     const int lnc0 = dm.layer_budgets ? st.n_layer[seq * dm.L + layer] : nc0;
-    if (half) lag_stream<LH, 1, true>(st, dm, kv, seq, 1, layer, threadIdx.x >> 7, lnc0);
-    else lag_stream<LH, 1>(st, dm, kv, seq, 1, layer, sidx & 1, lnc0);
+    if (half) lag_stream<LH, 1, true>(st, dm, kv, seq, 0, 1, 1, layer, threadIdx.x >> 7, lnc0);
+    else lag_stream<LH, 1>(st, dm, kv, seq, 0, 1, 1, layer, sidx & 1, lnc0);
   }
   __syncthreads();
   if (tid == 0) {
@@ -1046,6 +1124,34 @@ cudaError_t finalize_prepare() {
   allow(score_finalize_kernel<8>, mx);
   allow(score_finalize_kernel<32>, mx);
   return e;
+}
+
+#ifndef EPIKV_LAG_PIECE
+#define EPIKV_LAG_PIECE 128  // shortest piece (tokens); never under 8 chunks
+#endif
+#ifndef EPIKV_LAG_CTAS
+#define EPIKV_LAG_CTAS 56    // CTAs per SM wanted before pieces get longer: 8 rounds of 7 resident ones
+#endif
+// Tokens per piece of the K/V scoring kernel (lag_piece_start), 0 for one
+// piece per stream.  One CTA per (layer, K|V, sequence) leaves a call of few
+// sequences at one or two CTAs per SM, each a serial chain of loads: 4
+// prompts of 4,099 to 517 tokens, 32 layers, took 695 us (1.7 TB/s), all six
+// kinds of 2 prompts of 1,500 and 1,111 tokens 502 us.  Cut into pieces:
+// 231 us (5.2 TB/s) and 125 us.  A piece re-reads the chunk before it (L2),
+// so it has at least 8 chunks; 128 against 256 tokens 125 / 139 us on the
+// second call, and 7, 14, 28, 100 CTAs per SM 274, 247, 234, 224 us on the
+// first.  A call of less than two pieces stays whole (128 tokens of 32
+// sequences fill the GPU as they are).
+static int lag_piece_tokens(const Dims& dm, int n_seq, int max_new, int num_sms) {
+  const int64_t lag = dm.lag;
+  const int64_t least = (EPIKV_LAG_PIECE > 8 * lag ? (EPIKV_LAG_PIECE + lag - 1) / lag * lag : 8 * lag);
+  if (max_new < 2 * least) return 0;
+  const int64_t streams = (int64_t)2 * dm.L * n_seq, want = (int64_t)EPIKV_LAG_CTAS * num_sms;
+  const int64_t pieces = (want + streams - 1) / streams;
+  int64_t piece = (max_new + pieces - 1) / pieces;
+  piece = (piece + lag - 1) / lag * lag;
+  if (piece < least) piece = least;
+  return piece < max_new ? (int)piece : 0;
 }
 
 cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, const int32_t* seq_ids,
@@ -1110,24 +1216,32 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
     ++*launches;
   }
   if (dm.kinds & kKvKinds) {
-    const dim3 grid(2 * dm.L, n_seq);
+    const int piece = lag_piece_tokens(dm, n_seq, max_new, num_sms);
+    const dim3 grid(2 * dm.L, n_seq, lag_pieces(max_new, dm.lag, piece));
     const int threads = max(32, (dm.H * dm.d / 8 + 31) / 32 * 32);
-    auto go = [&](auto kern) { pdl_launch(kern, grid, threads, 0, stream, st, dm, *kv, seq_ids, cu_new, max_new); };
-    auto lanes = [&](auto kinds_t) {
+    auto go = [&](auto kern) {
+      pdl_launch(kern, grid, threads, 0, stream, st, dm, *kv, seq_ids, cu_new, max_new, piece);
+    };
+    auto lanes = [&](auto kinds_t, auto split_t) {
       constexpr int KS = decltype(kinds_t)::value;
+      constexpr bool SP = decltype(split_t)::value;
       switch (dm.d / 8) {
-        case 1: go(lagkv_partial_kernel<1, KS>); break;
-        case 2: go(lagkv_partial_kernel<2, KS>); break;
-        case 4: go(lagkv_partial_kernel<4, KS>); break;
-        case 8: go(lagkv_partial_kernel<8, KS>); break;
-        case 16: go(lagkv_partial_kernel<16, KS>); break;
-        default: go(lagkv_partial_kernel<32, KS>); break;
+        case 1: go(lagkv_partial_kernel<1, KS, SP>); break;
+        case 2: go(lagkv_partial_kernel<2, KS, SP>); break;
+        case 4: go(lagkv_partial_kernel<4, KS, SP>); break;
+        case 8: go(lagkv_partial_kernel<8, KS, SP>); break;
+        case 16: go(lagkv_partial_kernel<16, KS, SP>); break;
+        default: go(lagkv_partial_kernel<32, KS, SP>); break;
       }
     };
-    const int ks = ((dm.kinds & kNormKinds) ? 1 : 0) | ((dm.kinds & kRawKinds) ? 2 : 0);
-    if (ks == 1) lanes(std::integral_constant<int, 1>{});
-    else if (ks == 2) lanes(std::integral_constant<int, 2>{});
-    else lanes(std::integral_constant<int, 0>{});   // both: the runtime flags (fewer spills than both fixed)
+    auto kinds = [&](auto split_t) {
+      const int ks = ((dm.kinds & kNormKinds) ? 1 : 0) | ((dm.kinds & kRawKinds) ? 2 : 0);
+      if (ks == 1) lanes(std::integral_constant<int, 1>{}, split_t);
+      else if (ks == 2) lanes(std::integral_constant<int, 2>{}, split_t);
+      else lanes(std::integral_constant<int, 0>{}, split_t);   // both: the runtime flags (fewer spills than both fixed)
+    };
+    if (piece) kinds(std::true_type{});
+    else kinds(std::false_type{});
     ++*launches;
   }
   {
