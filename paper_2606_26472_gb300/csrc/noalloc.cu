@@ -41,9 +41,21 @@ namespace {
 
 constexpr size_t kNoallocScratchFloats = size_t(1) << 19;  // 2 MiB: n * 2 * num_layers floats
 constexpr int kMaxContexts = 64;  // contexts whose scratch address is remembered
-constexpr int kBatch = 16;
+constexpr int kSeg = 8;      // tokens per segment (never crosses a chunk boundary)
+constexpr int kOffs = 256;   // row offsets looked up together
 constexpr int kTile = 32;
 constexpr int kThreads = 256;
+constexpr int64_t kSms = 152;  // of a GB300
+#ifndef EPIKV_NOALLOC_CTAS
+#define EPIKV_NOALLOC_CTAS 14   // CTAs per SM wanted before pieces get longer: two rounds of 7 resident ones
+#endif
+#ifndef EPIKV_NOALLOC_CHUNKS
+#define EPIKV_NOALLOC_CHUNKS 2  // shortest piece
+#endif
+#ifndef EPIKV_NOALLOC_MAXREG
+#define EPIKV_NOALLOC_MAXREG 80  // measured best with 72 (128, 80, 72: 171, 128, 127 us on 4,001 tokens; 72 is slower on 200)
+#endif
+#define EPIKV_NOALLOC_BOUNDS __maxnreg__(EPIKV_NOALLOC_MAXREG)
 
 }  // namespace
 
@@ -53,88 +65,123 @@ namespace {
 
 using epikv::KvDev;
 
-// grid: 2L (layer, K|V); block: max(32, H*d/8) threads, d/8 lanes per head.
+// grid: (2L (layer, K|V), pieces of `piece` tokens, a multiple of lag);
+// block: max(32, H*d/8) threads, d/8 lanes per head, 8 channels each.
+//
+// A piece first takes the minimum and maximum of the chunk before it (bf16
+// values, kept packed; exact), so pieces are independent and one sequence
+// fills the GPU.  A call on 4,001 tokens of a 32-layer cache (524 MB) takes
+// 128 us (4.1 TB/s; bound by its instructions, two passes of arithmetic per
+// row), 200 tokens 19 us; one CTA per stream walking all tokens with a
+// butterfly per sum took 2,150 and 116 us.  Tokens are taken in segments of up
+// to 8 inside one chunk, their rows loaded together; the variance of a
+// token's head is taken in two passes over the normalised values, four tokens
+// at a time, their sums over the head's lanes by one transposed reduction.
+// part[stream][token]: neighbouring tokens' sums are stored, and later read,
+// together.
 template <int LH>
-__global__ void __launch_bounds__(256) noalloc_partial_kernel(KvDev kv, int seq, int n, int L, int H, int d,
-                                                              int lag, float lag_eps, float* part) {
+__global__ void EPIKV_NOALLOC_BOUNDS noalloc_partial_kernel(KvDev kv, int seq, int n, int L, int H, int d, int lag,
+                                                            float lag_eps, int piece, float* part) {
+  using namespace epikv;
   const int layer = blockIdx.x >> 1, kvk = blockIdx.x & 1;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31;
   const int h = tid / LH, q = tid % LH;
   const bool active = h < H;
   const int ch = h * d + q * 8;
-  float pmn[8], pmx[8], cmn[8], cmx[8], inv[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    pmn[e] = pmx[e] = cmn[e] = cmx[e] = 0.f;
-    inv[e] = 1.f / (pmx[e] - pmn[e] + lag_eps);
-  }
   const float inv_d = 1.f / (float)d;
-  const char* base = kv.base[kvk];
-  __shared__ float hv[kBatch][32];
-  for (int i0 = 0; i0 < n; i0 += kBatch) {
-    const int nbt = min(kBatch, n - i0);
-    uint4 x[kBatch];
+  const char* base = (kvk ? kv.base[1] : kv.base[0]) + (int64_t)ch * 2;
+  const int t_lo = blockIdx.y * piece, t_hi = min(n, t_lo + piece);
+  const int t_from = t_lo ? t_lo - lag : 0;   // the chunk before the piece: its range only
+  __shared__ int64_t soff[kOffs];
+  __shared__ float hv[2][kSeg][33];           // [parity][token][head]
+  uint4 cmn = make_uint4(0, 0, 0, 0), cmx = cmn;
+  f32x2 neg[4], inv[4];                       // -minimum and 1 / (maximum - minimum + eps) of the previous chunk
 #pragma unroll
-    for (int j = 0; j < kBatch; ++j) {
-      x[j] = make_uint4(0, 0, 0, 0);
-      if (j < nbt && active) {
-        const int64_t off = epikv::kv_row_offset(kv, layer, seq, i0 + j, n);
-        if (off >= 0) x[j] = epikv::ld_stream16(base + (off + ch) * 2);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < kBatch; ++j) {
-      if (j < nbt) {
-        const int pos = i0 + j;
-        const int c = pos / lag;
-        const int r = pos - c * lag;
-        float xf[8];
-        epikv::unpack8(x[j], xf);
-        float var = 0.f;
-        if (c >= 1) {
-          float xn[8], s = 0.f;
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            xn[e] = (xf[e] - pmn[e]) * inv[e];
-            s += xn[e];
-          }
-          const float mean = epikv::group_sum(s, LH) * inv_d;
-          float ss = 0.f;
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float dv = xn[e] - mean;
-            ss = fmaf(dv, dv, ss);
-          }
-          var = epikv::group_sum(ss, LH) * inv_d;
-        }
-        if (q == 0 && active) hv[j][h] = var;
-        if (r == 0) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) cmn[e] = cmx[e] = xf[e];
-        } else {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            cmn[e] = fminf(cmn[e], xf[e]);
-            cmx[e] = fmaxf(cmx[e], xf[e]);
-          }
-        }
-        if (r == lag - 1) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            pmn[e] = cmn[e];
-            pmx[e] = cmx[e];
-            inv[e] = 1.f / (pmx[e] - pmn[e] + lag_eps);
-          }
-        }
-      }
-    }
+  for (int p = 0; p < 4; ++p) neg[p] = inv[p] = 0ull;
+  int r = 0, parity = 0;                      // t_from is the first position of a chunk
+  for (int g0 = t_from; g0 < t_hi; g0 += kOffs) {
+    const int gn = min(kOffs, t_hi - g0);
     __syncthreads();
-    if (tid < nbt) {
-      float s = 0.f;
-      for (int hh = 0; hh < H; ++hh) s += hv[tid][hh];
-      part[(size_t)(i0 + tid) * (2 * L) + blockIdx.x] = s;
-    }
+    for (int t = tid; t < gn; t += blockDim.x) soff[t] = kv_row_offset(kv, layer, seq, g0 + t, n);
     __syncthreads();
+    for (int i = 0; i < gn;) {
+      const int seg = min(min(lag - r, gn - i), kSeg);
+      const int t0 = g0 + i;
+      const bool mine = t0 >= t_lo;           // a piece begins at a chunk, so never inside a segment
+      const bool score = mine && t0 >= lag;   // chunk 0 has no previous range: u = 0
+      uint4 x[kSeg];
+#pragma unroll
+      for (int j = 0; j < kSeg; ++j) {        // past the segment: its last row again, unused sums
+        const int64_t off = soff[i + min(j, seg - 1)];
+        x[j] = ld_stream16_if(base + off * 2, active && off >= 0);
+      }
+      if (r == 0) cmn = cmx = x[0];
+#pragma unroll
+      for (int j = 0; j < kSeg; j += 2) {
+        cmn = q_min(q_min(cmn, x[j]), x[j + 1]);
+        cmx = q_max(q_max(cmx, x[j]), x[j + 1]);
+      }
+      if (score) {
+#pragma unroll
+        for (int j0 = 0; j0 < kSeg; j0 += 4) {
+          f32x2 y[4][4];
+          float v[4], tot[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t w[4] = {x[j0 + j].x, x[j0 + j].y, x[j0 + j].z, x[j0 + j].w};
+#pragma unroll
+            for (int p = 0; p < 4; ++p) y[j][p] = f2_mul(f2_add(bf16x2_to_f2(w[p]), neg[p]), inv[p]);
+            const f32x2 s = f2_add(f2_add(y[j][0], y[j][1]), f2_add(y[j][2], y[j][3]));
+            v[j] = f2_lo(s) + f2_hi(s);
+          }
+          group_totals<LH>(v, lane, tot);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float m = -tot[j] * inv_d;
+            const f32x2 nm = f2_pack(m, m);
+            f32x2 ss = 0ull;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+              const f32x2 dv = f2_add(y[j][p], nm);
+              ss = f2_fma(dv, dv, ss);
+            }
+            v[j] = f2_lo(ss) + f2_hi(ss);
+          }
+          transpose_sum<LH / 2, 4, 4>(v, lane);
+          if (active) {
+            if constexpr (LH <= 4) {
+#pragma unroll
+              for (int k = 0; k < 4 / LH; ++k) hv[parity][j0 + k + (4 / LH) * q][h] = v[k];
+            } else {
+              if (q % (LH / 4) == 0) hv[parity][j0 + q / (LH / 4)][h] = v[0];
+            }
+          }
+        }
+      }
+      if (mine) {
+        __syncthreads();   // hv is double buffered: one barrier per segment
+        if (tid < seg) {
+          float s = 0.f;
+          if (score)
+            for (int hh = 0; hh < H; ++hh) s += hv[parity][tid][hh];
+          part[(size_t)blockIdx.x * n + t0 + tid] = s * inv_d;
+        }
+        parity ^= 1;
+      }
+      r += seg;
+      if (r == lag) {      // the chunk is complete: it becomes the previous one
+        float mn[8], mx[8];
+        unpack8(cmn, mn);
+        unpack8(cmx, mx);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          neg[p] = f2_pack(-mn[2 * p], -mn[2 * p + 1]);
+          inv[p] = f2_pack(__frcp_rn(mx[2 * p] - mn[2 * p] + lag_eps), __frcp_rn(mx[2 * p + 1] - mn[2 * p + 1] + lag_eps));
+        }
+        r = 0;
+      }
+      i += seg;
+    }
   }
 }
 
@@ -142,6 +189,7 @@ __global__ void __launch_bounds__(256) noalloc_partial_kernel(KvDev kv, int seq,
 template <int WPL>
 __global__ void __launch_bounds__(kThreads) noalloc_finalize_kernel(const float* part, int n, int L, int H, int lag,
                                                                     int w, float* out) {
+  epikv::pdl_wait();
   __shared__ float su[kTile + 1024];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int i_lo = blockIdx.x * kTile, i_hi = min(i_lo + kTile, n);
@@ -150,9 +198,9 @@ __global__ void __launch_bounds__(kThreads) noalloc_finalize_kernel(const float*
   for (int i = lo + tid; i < i_hi; i += kThreads) {
     float u = 0.f;
     if (i >= lag) {
-      const float* pp = part + (size_t)i * (2 * L);
       float s = 0.f;
-      for (int q = 0; q < 2 * L; ++q) s += pp[q];
+#pragma unroll 16
+      for (int q = 0; q < 2 * L; ++q) s += part[(size_t)q * n + i];
       u = s * inv_lh;
     }
     su[i - lo] = u;
@@ -169,6 +217,18 @@ __global__ void __launch_bounds__(kThreads) noalloc_finalize_kernel(const float*
     const float mean = epikv::warp_sum(acc) / (float)cnt;
     if (lane == 0) out[i] = mean;
   }
+}
+
+// Tokens per piece: as long as there are EPIKV_NOALLOC_CTAS CTAs per SM, since
+// a piece re-reads (from L2) the chunk before it, and at least two chunks
+// (4,001 / 200 tokens: 7 CTAs per SM 141 / 19 us, 14 128 / 19, 28 130 / 19; at
+// least four chunks 130 / 24).
+int piece_tokens(int n, int L, int lag) {
+  const int64_t least = (int64_t)EPIKV_NOALLOC_CHUNKS * lag, streams = 2 * (int64_t)L;
+  const int64_t pieces = (EPIKV_NOALLOC_CTAS * kSms + streams - 1) / streams;
+  int64_t piece = ((n + pieces - 1) / pieces + lag - 1) / lag * lag;
+  if (piece < least) piece = least;
+  return piece < n ? (int)piece : n;
 }
 
 // The current context's unique id (driver entry points fetched through the
@@ -276,27 +336,26 @@ extern "C" epikv_status epikv_lagkv_score_noalloc(const epikv_kv_view* kv, int32
   if (scratch_address(&part) != cudaSuccess) return EPIKV_ECUDA;
 
   const int threads = (H * d / 8 + 31) / 32 * 32 < 32 ? 32 : (H * d / 8 + 31) / 32 * 32;
-  const dim3 g1(2 * L);
+  const int piece = piece_tokens(n, L, lag);
+  const dim3 g1(2 * L, (n + piece - 1) / piece);
   switch (d / 8) {
-    case 1: noalloc_partial_kernel<1><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, part); break;
-    case 2: noalloc_partial_kernel<2><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, part); break;
-    case 4: noalloc_partial_kernel<4><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, part); break;
-    case 8: noalloc_partial_kernel<8><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, part); break;
-    case 16: noalloc_partial_kernel<16><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, part); break;
-    default: noalloc_partial_kernel<32><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, part); break;
+    case 1: noalloc_partial_kernel<1><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, piece, part); break;
+    case 2: noalloc_partial_kernel<2><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, piece, part); break;
+    case 4: noalloc_partial_kernel<4><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, piece, part); break;
+    case 8: noalloc_partial_kernel<8><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, piece, part); break;
+    case 16: noalloc_partial_kernel<16><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, piece, part); break;
+    default: noalloc_partial_kernel<32><<<g1, threads, 0, stream>>>(kd, seq, n, L, H, d, lag, lag_eps, piece, part); break;
   }
   const dim3 g2((n + kTile - 1) / kTile);
   const int wpl = (window + 31) / 32;
-  if (wpl <= 1)
-    noalloc_finalize_kernel<1><<<g2, kThreads, 0, stream>>>(part, n, L, H, lag, window, d_scores);
-  else if (wpl <= 2)
-    noalloc_finalize_kernel<2><<<g2, kThreads, 0, stream>>>(part, n, L, H, lag, window, d_scores);
-  else if (wpl <= 4)
-    noalloc_finalize_kernel<4><<<g2, kThreads, 0, stream>>>(part, n, L, H, lag, window, d_scores);
-  else if (wpl <= 8)
-    noalloc_finalize_kernel<8><<<g2, kThreads, 0, stream>>>(part, n, L, H, lag, window, d_scores);
-  else
-    noalloc_finalize_kernel<32><<<g2, kThreads, 0, stream>>>(part, n, L, H, lag, window, d_scores);
+  auto fin = [&](auto kern) {
+    epikv::pdl_launch(kern, g2, dim3(kThreads), 0, stream, (const float*)part, n, L, H, lag, window, d_scores);
+  };
+  if (wpl <= 1) fin(noalloc_finalize_kernel<1>);
+  else if (wpl <= 2) fin(noalloc_finalize_kernel<2>);
+  else if (wpl <= 4) fin(noalloc_finalize_kernel<4>);
+  else if (wpl <= 8) fin(noalloc_finalize_kernel<8>);
+  else fin(noalloc_finalize_kernel<32>);
   // no error was pending before the launches, so any error now is theirs
   return cudaGetLastError() == cudaSuccess ? EPIKV_OK : EPIKV_ECUDA;
 }

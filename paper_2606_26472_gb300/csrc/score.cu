@@ -186,55 +186,6 @@ constexpr int kLagSeg = EPIKV_LAG_SEG;  // tokens per segment (never crosses a c
 constexpr int kLagPf = EPIKV_LAG_PF;    // a row is prefetched into L2 this many segments ahead
 constexpr int kLagOffs = 256;   // slot offsets looked up per group of tokens
 
-// Fire-and-forget bulk prefetch of [p, p + bytes) into L2 (p 16-byte aligned,
-// bytes a multiple of 16).
-__device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ uint32_t bf16x2_min(uint32_t a, uint32_t b) {
-  __nv_bfloat162 r = __hmin2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
-  return *reinterpret_cast<uint32_t*>(&r);
-}
-__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
-  __nv_bfloat162 r = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
-  return *reinterpret_cast<uint32_t*>(&r);
-}
-__device__ __forceinline__ uint4 q_min(const uint4& a, const uint4& b) {
-  return make_uint4(bf16x2_min(a.x, b.x), bf16x2_min(a.y, b.y), bf16x2_min(a.z, b.z), bf16x2_min(a.w, b.w));
-}
-__device__ __forceinline__ uint4 q_max(const uint4& a, const uint4& b) {
-  return make_uint4(bf16x2_max(a.x, b.x), bf16x2_max(a.y, b.y), bf16x2_max(a.z, b.z), bf16x2_max(a.w, b.w));
-}
-
-// ---- packed fp32 pairs: Blackwell's f32x2 arithmetic, two channels per instruction
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
-  f32x2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-  return d;
-}
-__device__ __forceinline__ float f2_lo(f32x2 v) { return __uint_as_float((unsigned)(v & 0xffffffffull)); }
-__device__ __forceinline__ float f2_hi(f32x2 v) { return __uint_as_float((unsigned)(v >> 32)); }
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-// the two bf16 channels of a 32-bit word as an fp32 pair (exact)
-__device__ __forceinline__ f32x2 bf16x2_to_f2(uint32_t w) { return f2_pack(bf16_lo(w), bf16_hi(w)); }
-
 // The previous chunk's range as a per-channel affine map y = x * a + c with
 // a = 1 / (max - min + eps) and c = -min * a - 1/2, so that y = x~ - 1/2 for
 // the range-normalised x~ (one fused multiply-add per channel).
@@ -269,31 +220,6 @@ __device__ __forceinline__ void lag_moments(const uint4& x, const f32x2 (&a)[4],
   u = f2_fma(y3, y3, u);
   s1 = f2_lo(t) + f2_hi(t);
   s2 = f2_lo(u) + f2_hi(u);
-}
-
-// Transposed sum over the O*2 lanes of a group: every level halves the values
-// a lane keeps and sends the other half to its partner, so NV values cost
-// NV - 1 shuffles in all instead of one butterfly of log2(lanes) shuffles per
-// value.  With lanes <= NV, value k + (NV / lanes) * (lane % lanes) ends in
-// v[k]; with more lanes than values, value (lane % lanes) / (lanes / NV) ends
-// in v[0].
-template <int O, int C, int NV>
-__device__ __forceinline__ void transpose_sum(float (&v)[NV], int lane) {
-  if constexpr (O >= 1) {
-    if constexpr (C > 1) {
-      const bool up = lane & O;
-#pragma unroll
-      for (int k = 0; k < C / 2; ++k) {
-        const float send = up ? v[k] : v[k + C / 2];
-        const float keep = up ? v[k + C / 2] : v[k];
-        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-      }
-      transpose_sum<O / 2, C / 2, NV>(v, lane);
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-      transpose_sum<O / 2, 1, NV>(v, lane);
-    }
-  }
 }
 
 // grid: (2L (layer, K|V), batch entries); block: max(32, H*d/8) threads;
