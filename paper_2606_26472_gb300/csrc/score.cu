@@ -390,9 +390,50 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
           const int t = i + kLagPf * SEG + tid;
           if (tid < seg && t < gn && soff[t] >= 0) prefetch_l2_bulk(kvbase + soff[t] * 2, row_bytes);
         }
+        // the raw kinds, four tokens at a time (absent ones give unused
+        // sums): population variances of the stored vectors over the head
+        // dimension, two transposed reductions instead of eight butterflies
+        if constexpr (SEG % 4 == 0) {
+          if (need_raw) {
+#pragma unroll
+            for (int j0 = 0; j0 < SEG; j0 += 4) {
+              float rv[4], tot[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                float xf[8], s1 = 0.f;
+                unpack8(x[j0 + j], xf);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) s1 += xf[e];
+                rv[j] = s1;
+              }
+              group_totals<LH>(rv, tid & 31, tot);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                float xf[8], s2 = 0.f;
+                unpack8(x[j0 + j], xf);
+                const float mean = tot[j] * inv_d;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  const float dv = xf[e] - mean;
+                  s2 = fmaf(dv, dv, s2);
+                }
+                rv[j] = s2;
+              }
+              transpose_sum<LH / 2, 4, 4>(rv, tid & 31);
+              if (active) {
+                if constexpr (LH <= 4) {
+#pragma unroll
+                  for (int k = 0; k < 4 / LH; ++k) hr[parity][j0 + k + (4 / LH) * q][h] = rv[k] * inv_d;
+                } else {
+                  if (q % (LH / 4) == 0) hr[parity][j0 + q / (LH / 4)][h] = rv[0] * inv_d;
+                }
+              }
+            }
+          }
+        }
         // two tokens at a time, so that rows' registers are free once used:
-        // their raw variances, their normalised moments, then the running
-        // range over both (the same min/max sequence as token by token)
+        // their normalised moments, then the running range over both (the
+        // same min/max sequence as token by token)
         float v[NV];
         if (r == 0) {
           cmn = x[0];
@@ -403,7 +444,7 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
 #pragma unroll
           for (int j = j0; j < j0 + 2 && j < SEG; ++j) {
             if (FULL || j < seg) {
-              if (need_raw) {  // population variance of the stored vector over the head dimension
+              if (SEG % 4 != 0 && need_raw) {  // population variance of the stored vector over the head dimension
                 float xf[8], s1 = 0.f;
                 unpack8(x[j], xf);
 #pragma unroll
@@ -504,8 +545,16 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
 #ifndef EPIKV_LAG_MAXREG
 #define EPIKV_LAG_MAXREG 72  // 7 CTAs of 128 threads per SM: 2,048 CTAs in two rounds (measured best; 64 spills)
 #endif
+#ifndef EPIKV_LAG_RAWREG
+// with the raw kinds: 96, five CTAs per SM.  Prompts of 1,500 and 1,111 tokens,
+// 32 layers, at 72 / 80 / 96 / 128 registers: the raw kinds alone 67 / 66 / 62
+// / 79 us (342 MB: 5.5 TB/s), all K/V kinds 135 / 126 / 109 / 119 us (72 and
+// 80 spill); 125 us for all with a butterfly per sum instead of the
+// transposed reductions
+#define EPIKV_LAG_RAWREG 96
+#endif
 #if EPIKV_LAG_MAXREG > 0
-#define EPIKV_LAG_BOUNDS __maxnreg__(EPIKV_LAG_MAXREG)
+#define EPIKV_LAG_BOUNDS __maxnreg__(KINDS == 1 ? EPIKV_LAG_MAXREG : EPIKV_LAG_RAWREG)
 #else
 #define EPIKV_LAG_BOUNDS __launch_bounds__(256, EPIKV_LAG_MINB)
 #endif
@@ -1164,7 +1213,7 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
       const int ks = ((dm.kinds & kNormKinds) ? 1 : 0) | ((dm.kinds & kRawKinds) ? 2 : 0);
       if (ks == 1) lanes(std::integral_constant<int, 1>{}, split_t);
       else if (ks == 2) lanes(std::integral_constant<int, 2>{}, split_t);
-      else lanes(std::integral_constant<int, 0>{}, split_t);   // both: the runtime flags (fewer spills than both fixed)
+      else lanes(std::integral_constant<int, 0>{}, split_t);   // both: the runtime flags (109 us, both fixed 168)
     };
     if (piece) kinds(std::true_type{});
     else kinds(std::false_type{});
