@@ -49,8 +49,8 @@ struct DevState {
   float* g_ring;           // [S][n_band][G] g by position (mod G)
   float* ztok;             // [S][2][n_band] a decode step's per-band z and window mean of g (band kinds)
   __nv_bfloat16* lag_rng;  // [S][L][2][4][H][d] prev min, prev max, cur min, cur max
-  float* lag_part;         // [S][max_new][2L] per-(layer, K|V) head-summed normalised variances
-  float* raw_part;         // [S][max_new][2L] per-(layer, K|V) head-summed raw variances
+  float* lag_part;         // [S][2L][max_new] per-(layer, K|V) head-summed normalised variances (a decode step: [S][2L] at the front)
+  float* raw_part;         // the same of the raw variances
   float* u_ring[4];        // [S][G] per K/V kind (kv_kind order): u by position (mod G)
   int32_t* kept;           // [S][T] kept lists of epikv_step
   int32_t* n_kept;         // [S]

@@ -331,6 +331,10 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
   float (*hr)[SEG][32] = hr_s[half];
   float* part = need_norm ? st.lag_part + (size_t)seq * dm.max_new * (2 * dm.L) : nullptr;
   float* rpart = need_raw ? st.raw_part + (size_t)seq * dm.max_new * (2 * dm.L) : nullptr;
+  // this stream's partials: [stream][token], so that neighbouring tokens'
+  // lie together for score_finalize_kernel; a decode step's one token
+  // [stream], for kv_token_scores
+  const size_t part0 = SEG == 1 ? (size_t)stream : (size_t)stream * dm.max_new;
   int r = (p0 + t_lo) % dm.lag;          // position of the next token inside its chunk
   int parity = 0;
 
@@ -500,12 +504,12 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
               const float mean = red[parity][hh][2 * tid] * inv_d;
               sum += fmaxf(fmaf(-mean, mean, red[parity][hh][2 * tid + 1] * inv_d), 0.f);
             }
-          part[(size_t)(g0 + i + tid) * (2 * dm.L) + stream] = sum;
+          part[part0 + g0 + i + tid] = sum;
         }
         if (need_raw) {
           float sum = 0.f;
           for (int hh = 0; hh < dm.H; ++hh) sum += hr[parity][tid][hh];
-          rpart[(size_t)(g0 + i + tid) * (2 * dm.L) + stream] = sum;
+          rpart[part0 + g0 + i + tid] = sum;
         }
       }
       parity ^= 1;
@@ -636,6 +640,7 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
   const int Gm = dm.G - 1;
   const int nb = dm.nA + dm.nB;
 
+  extern __shared__ float sg[];  // band kinds: [nb][span] windows of g; then the K/V kinds' u
   if (fits && i_lo < i_hi) {
     for (int i = i_lo + warp; i < i_hi; i += kFinThreads / 32) {
       const int pos = p0 + i;
@@ -645,7 +650,6 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
     }
     if (dm.kinds & kBandKinds) {
       // every g value the tile's windows reach, all band layers, one round of loads
-      extern __shared__ float sg[];  // [nb][span]
       const int span = kFinTile + dm.z_window - 1;
       const int pos_base = p0 + i_lo - (dm.z_window - 1);  // position held by sg[band][0]
       const int pos_end = p0 + i_hi;
@@ -703,46 +707,59 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
       }
     }
     if (dm.kinds & kKvKinds) {
-      __shared__ float su[kFinTile + kMaxWindow];
+      // u of the tile's tokens and their windows' earlier ones in this call,
+      // a thread per (kind, token), every kind's loads in flight together and
+      // neighbouring threads' loads side by side (partials [stream][token]):
+      // 4 prompts of 4,099 to 517 tokens 18 us, [token][stream] 23.5 us; all
+      // six kinds of 1,500 and 1,111 tokens 24 us, one kind after another 31 us
+      float* su = sg + (dm.kinds & kBandKinds ? nb * (kFinTile + dm.z_window - 1) : 0);  // [kind][lo .. i_hi)
       const int w = dm.lag_window;
       const int lo = max(0, i_lo - (w - 1));
+      const int cnt = i_hi - lo, tile = i_hi - i_lo;
       const float inv_lh = 1.f / (float)(dm.L * dm.H);
-      for (int qk = 0; qk < 4; ++qk) {
-        const int kind = kv_kind(qk);
-        if (!(dm.kinds & kind)) continue;
+      const int nk = __popc(dm.kinds & kKvKinds);
+      auto nth_kind = [&](int c) -> int {  // the c-th K/V kind held, in kv_kind order
+        int qk = 0;
+        for (int left = c;; ++qk)
+          if ((dm.kinds & kv_kind(qk)) && left-- == 0) return qk;
+      };
+      for (int idx = tid; idx < nk * cnt; idx += kFinThreads) {
+        const int c = idx / cnt, i = lo + (idx - c * cnt);
+        const int kind = kv_kind(nth_kind(c));
         // which partials: normalised or raw; all (layer, K|V) entries, keys only or values only
         const bool raw = kind & kRawKinds;
-        const float* part = (raw ? st.raw_part : st.lag_part) + (size_t)seq * dm.max_new * (2 * dm.L);
+        const float* pp = (raw ? st.raw_part : st.lag_part) + (size_t)seq * dm.max_new * (2 * dm.L) + i;
         const int q0 = kind == EPIKV_SCORE_KVVAL ? 1 : 0;
         const int qs = kind == EPIKV_SCORE_LAGKV ? 1 : 2;
-        float* ring = st.u_ring[qk] + (size_t)seq * dm.G;
-        float* out = st.score[kind_index(kind)] + (size_t)seq * dm.T + nc0;
-        __syncthreads();  // su is reused kind after kind
-        for (int i = lo + tid; i < i_hi; i += kFinThreads) {
-          const int pos = p0 + i;
-          float u = 0.f;
-          if (raw || pos >= dm.lag) {  // the normalised kinds have no value in chunk 0
-            const float* pp = part + (size_t)i * (2 * dm.L);
-            float s = 0.f;
-            for (int q = q0; q < 2 * dm.L; q += qs) s += pp[q];
-            u = s * inv_lh;
-          }
-          su[i - lo] = u;
+        float u = 0.f;
+        if (raw || p0 + i >= dm.lag) {  // the normalised kinds have no value in chunk 0
+          float s = 0.f;
+#pragma unroll 16
+          for (int q = q0; q < 2 * dm.L; q += qs) s += pp[(size_t)q * dm.max_new];
+          u = s * inv_lh;
         }
-        __syncthreads();
-        for (int i = i_lo + warp; i < i_hi; i += kFinThreads / 32) {
-          const int pos = p0 + i;
-          const int n = min(w, pos + 1);
-          float acc = 0.f;
+        su[idx] = u;
+      }
+      __syncthreads();
+      for (int it = warp; it < nk * tile; it += kFinThreads / 32) {
+        const int c = it / tile, i = i_lo + (it - c * tile);
+        const int qk = nth_kind(c);
+        const float* ring = st.u_ring[qk] + (size_t)seq * dm.G;
+        const float* us = su + c * cnt - lo;
+        const int pos = p0 + i;
+        const int n = min(w, pos + 1);
+        float acc = 0.f;
 #pragma unroll
-          for (int m = 0; m < WPL; ++m) {
-            const int k = lane + 32 * m;
-            if (k < n) acc += (i - k >= 0) ? su[i - k - lo] : ring[(pos - k) & Gm];
-          }
-          const float mean = warp_sum(acc) / (float)n;
-          if (lane == 0) out[i] = mean;
+        for (int m = 0; m < WPL; ++m) {
+          const int k = lane + 32 * m;
+          if (k < n) acc += (i - k >= 0) ? us[i - k] : ring[(pos - k) & Gm];
         }
-        for (int i = i_lo + tid; i < i_hi; i += kFinThreads) ring[(p0 + i) & Gm] = su[i - lo];
+        const float mean = warp_sum(acc) / (float)n;
+        if (lane == 0) st.score[kind_index(kv_kind(qk))][(size_t)seq * dm.T + nc0 + i] = mean;
+      }
+      for (int it = tid; it < nk * tile; it += kFinThreads) {
+        const int c = it / tile, i = i_lo + (it - c * tile);
+        st.u_ring[nth_kind(c)][(size_t)seq * dm.G + ((p0 + i) & Gm)] = su[c * cnt + i - lo];
       }
     }
   }
@@ -1072,13 +1089,16 @@ __global__ void __launch_bounds__(kGThreads, EPIKV_TOKEN_MINB) token_kernel(DevS
 
 // ------------------------------------------------------------------ launchers
 // dynamic shared memory of the finalize kernel: the band windows of a tile
+// and the K/V kinds' u over it
 static size_t finalize_smem(const Dims& dm) {
-  if (!(dm.kinds & kBandKinds)) return 0;
-  return (size_t)(dm.nA + dm.nB) * (kFinTile + dm.z_window - 1) * sizeof(float);
+  size_t words = 0;
+  if (dm.kinds & kBandKinds) words += (size_t)(dm.nA + dm.nB) * (kFinTile + dm.z_window - 1);
+  words += (size_t)__builtin_popcount((unsigned)(dm.kinds & kKvKinds)) * (kFinTile + dm.lag_window - 1);
+  return words * sizeof(float);
 }
 
 cudaError_t finalize_prepare() {
-  const int mx = (int)((size_t)kMaxBand * (kFinTile + kMaxWindow - 1) * sizeof(float));
+  const int mx = (int)((size_t)(kMaxBand + 4) * (kFinTile + kMaxWindow - 1) * sizeof(float));
   const int wmx = (int)((size_t)kMaxBand * kMaxWindow * sizeof(float));
   cudaError_t e = cudaSuccess;
   auto allow = [&](auto kern, int bytes) {
