@@ -153,8 +153,7 @@ inline cudaError_t pdl_launch(void (*kernel)(Params...), dim3 grid, dim3 block, 
   return launch_kernel(true, kernel, grid, block, smem, stream, args...);
 }
 
-// Plain stream order: the long copy kernel, whose CTAs spread more evenly
-// when none of them is placed before the kernel ahead of it has finished.
+// Plain stream order: the copy kernel where no stash kernel runs before it.
 template <typename... Params, typename... Args>
 inline cudaError_t plain_launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                                 Args... args) {

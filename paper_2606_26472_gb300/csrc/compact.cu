@@ -75,6 +75,13 @@ constexpr int kStagedBlocks = EPIKV_COMPACT_STAGED_BLOCKS;
 
 constexpr int kStashThreads = 512;
 constexpr int kStashUnroll = 4;
+// Bytes moved (read and written) up to which the copy's CTAs are let in while
+// the stash kernel runs, instead of as its CTAs end.  It hides the launch and
+// the copy's own look-up of its rows, but CTAs placed early copy 1.3 % slower
+// over a long copy: 0.13 GB 55.5 us per step early / 58.2 late (60.5 without
+// programmatic launch), 1.2 GB 240.5 / 241.5 (246.5), 8.4 GB 1,359 / 1,342
+// (1,342), 67 GB 10,400 / 10,250 (10,250).
+constexpr int64_t kStashEarlyBytes = 1ll << 30;
 
 // The balanced split's row space is made of pairs: under token budgets one
 // per evicting entry, with its 2L streams; under per-layer budgets one per
@@ -252,9 +259,15 @@ struct Cursor {
 template <bool kLayers, bool kSplit>
 __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev kv,
                                                      const int32_t* __restrict__ seq_ids, int n_seq,
-                                                     const int32_t* __restrict__ kept, int kept_stride) {
-  pdl_wait();
-  pdl_trigger();
+                                                     const int32_t* __restrict__ kept, int kept_stride,
+                                                     int after_stash) {
+  // Launched programmatically after compact_stash_kernel (after_stash), the
+  // CTAs start beside it: that kernel lets them in only after its own wait,
+  // so the selection's results are complete, and it writes neither those nor
+  // the cache.  What it writes, the stash, and what it still reads, the rows
+  // this kernel overwrites, are first touched after the wait below.
+  bool waited = !(kSplit && after_stash);
+  if (waited) pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t full[kStages];
   __shared__ char* dptr[kStages][kMaxRPB];
@@ -267,7 +280,10 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
 
   // ---- the batch entries that evicted (every CTA builds the same list)
   const int n_ev = evicting_entries(st, dm, seq_ids, n_seq, list, kLayers ? nullptr : pre, lane);
-  if (n_ev == 0) return;
+  if (n_ev == 0) {
+    pdl_wait();   // this kernel ends after the stash kernel, for the kernels that wait for this one
+    return;
+  }
   // ---- the balanced split's pairs and their rows
   const int n_pairs = kLayers ? n_ev * dm.L : n_ev;
   const int sp = kLayers ? 2 : 2 * dm.L;  // streams per pair
@@ -366,7 +382,7 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
       c.end = c.i + (int)(o_stop - o);
       c.stash_at = c.end;
       c.n_new = a.n_new;
-      c.row0 = st.stash_row0[blockIdx.x + 1];            // written by compact_stash_kernel
+      c.row0 = st.stash_row0[blockIdx.x + 1];            // written by compact_stash_kernel (read again after the wait)
     } else {
       c.end = c.i + (int)rest;
       c.stash_at = INT_MAX;
@@ -476,12 +492,27 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   prefetch(ld, pk);
   int k_issue = 0, k_store = 0;
   bool timed_out = false;
+  // the first loads go out before the wait, up to a batch with rows that
+  // come from the stash
+  auto wait_stash = [&] {
+    pdl_wait();
+    waited = true;
+    if (ld.u < units && ld.stash_at != INT_MAX) ld.row0 = st.stash_row0[blockIdx.x + 1];
+  };
   for (int p = 0; p < kStages - 1 && ld.u < units; ++p) {
+    if (!waited) {
+      bool stashed = false;
+#pragma unroll
+      for (int j = 0; j < kMaxRowsPerLane; ++j) stashed |= pk[j] >= ld.stash_at;
+      if (__any_sync(0xffffffffu, stashed)) wait_stash();
+    }
     issue(ld, pk, k_issue % kStages);
     ++k_issue;
     advance(ld);
     prefetch(ld, pk);
   }
+  if (!waited) wait_stash();
+  pdl_trigger();
   while (k_store < k_issue) {
     const int s = k_store % kStages;
     if (!mbar_wait_bounded(&full[s], (k_store / kStages) & 1, kWaitNs)) {
@@ -531,7 +562,6 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
                                                                       int n_seq, const int32_t* __restrict__ kept,
                                                                       int kept_stride) {
   pdl_wait();
-  pdl_trigger();
   extern __shared__ __align__(128) unsigned char smem[];
   int* list = reinterpret_cast<int*>(smem);
   int64_t* pre = reinterpret_cast<int64_t*>(list + list_ints(n_seq));
@@ -555,9 +585,11 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
     }
   }
   __syncthreads();
+  const int64_t total = s_rows * sp;
+  // compact_kernel's CTAs are let in now, or as this kernel ends (kStashEarlyBytes)
+  if (total * dm.H * dm.d * 4 <= kStashEarlyBytes) pdl_trigger();
   if (!s_bal || blockIdx.x == 0) return;
   const int n_pairs = s_pairs;
-  const int64_t total = s_rows * sp;
   const int64_t o = (int64_t)blockIdx.x * total / gridDim.x;
   if (o >= total) return;
   int p, q;
@@ -621,12 +653,17 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
 
 // The batch entries' evictions have been applied: nothing is left pending.
 __global__ void compact_consumed_kernel(DevState st, Dims dm, const int32_t* __restrict__ seq_ids, int n_seq) {
+  // launched beside the copy, which does not write the lengths: they are
+  // loaded before the wait
+  const int b0 = blockIdx.x * blockDim.x + threadIdx.x;
+  const int seq0 = b0 < n_seq ? seq_ids[b0] : -1;
+  const int n0 = seq0 >= 0 && seq0 < dm.S ? st.n_cache[seq0] : 0;
   pdl_wait();
   pdl_trigger();
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n_seq; b += gridDim.x * blockDim.x) {
-    const int seq = seq_ids[b];
+  for (int b = b0; b < n_seq; b += gridDim.x * blockDim.x) {
+    const int seq = b == b0 ? seq0 : seq_ids[b];
     if (seq < 0 || seq >= dm.S) continue;
-    st.first_changed[seq] = st.n_cache[seq];
+    st.first_changed[seq] = b == b0 ? n0 : st.n_cache[seq];
     if (dm.layer_budgets)
       for (int l = 0; l < dm.L; ++l) st.lfirst[seq * dm.L + l] = st.n_layer[seq * dm.L + l];
   }
@@ -673,7 +710,8 @@ cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const 
   const bool layers = dm.layer_budgets;
   const bool split = !layers || n_seq * dm.L <= kMaxLayerPairs;  // the balanced split may apply
   const size_t smem = compact_smem(n_seq, dm.L, layers);
-  if (split && ctas <= kMaxStashCtas) {  // the balanced split's stash (the kernel checks whether it applies)
+  const bool stash = split && ctas <= kMaxStashCtas;
+  if (stash) {  // the balanced split's stash (the kernel checks whether it applies)
     pdl_launch(compact_stash_kernel, ctas, kStashThreads, stash_smem(n_seq, dm.L, layers), stream, st, dm, kv,
                seq_ids, n_seq, kept, kept_stride);
     ++*launches;
@@ -681,7 +719,10 @@ cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const 
     if (e != cudaSuccess) return e;
   }
   auto go = [&](auto kern) {
-    plain_launch(kern, ctas, 32, smem, stream, st, dm, kv, seq_ids, n_seq, kept, kept_stride);
+    if (stash)
+      pdl_launch(kern, ctas, 32, smem, stream, st, dm, kv, seq_ids, n_seq, kept, kept_stride, 1);
+    else
+      plain_launch(kern, ctas, 32, smem, stream, st, dm, kv, seq_ids, n_seq, kept, kept_stride, 0);
   };
   if (!layers) go(compact_kernel<false, true>);
   else if (split) go(compact_kernel<true, true>);
