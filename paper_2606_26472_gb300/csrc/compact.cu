@@ -32,8 +32,20 @@
 // copies those rows aside before the compaction starts, and the chunk reads
 // them there.  They are a suffix of the chunk's rows in that stream, no
 // longer than the chunk nor than the eviction's largest shift
-// kept[n-1] - (n-1); when both bounds exceed the stash, the per-stream units
-// above are used instead.
+// kept[n-1] - (n-1).
+//
+// Head and tail split (token budgets, when both bounds exceed the stash): rows
+// from the first one whose source lies at or past the new length, the tail,
+// read slots that no row is written to.  compact_stash_kernel moves the rows
+// before it, the head, in place, a CTA per (stream, head group) in increasing
+// row order; the copy then moves every tail, one equal chunk per CTA, with no
+// row in any chunk's way.  Cutting n slots to K at random leaves about K * K /
+// n rows in the head.  A batch of many streams whose heads are long keeps the
+// per-stream units.  32 layers, 2 KiB rows, units (with their 512-byte to 1
+// KiB pieces) / head + tail: 65,536, 38,940 and 12,345 slots to 4,096 (3.2 GB
+// moved) 850 / 90 + 461 us; 9,000 to 3,000 461 / 52 + 97; 3 x 8,192 to 4,096
+// 847 / 272 + 289 (half the rows are in the heads, at 6 TB/s); 4,396 to 4,096
+// (nearly all in the head) 575 / 167 + 22.
 //
 // A selection's eviction is compacted once: compact_consumed_kernel, launched
 // after the copy, sets each sequence's first moved slot to its length, so
@@ -82,6 +94,9 @@ constexpr int kStashUnroll = 4;
 // programmatic launch), 1.2 GB 240.5 / 241.5 (246.5), 8.4 GB 1,359 / 1,342
 // (1,342), 67 GB 10,400 / 10,250 (10,250).
 constexpr int64_t kStashEarlyBytes = 1ll << 30;
+constexpr int kHeadUnroll = 8;        // vectors per thread and batch of the head
+constexpr int kMaxHeadRows = 512;     // rows per batch of the head
+constexpr int64_t kUnitRounds = 4;    // streams per CTA from which per-stream units are even enough
 
 // The balanced split's row space is made of pairs: under token budgets one
 // per evicting entry, with its 2L streams; under per-layer budgets one per
@@ -224,6 +239,58 @@ __device__ bool balanced_split(const DevState& st, const Dims& dm, const int32_t
   return __all_sync(0xffffffffu, ok);
 }
 
+// The first row in [first, n_new) of a kept list whose source is at or past
+// n_new (n_new if none): an eight-way search, its probes loaded together.
+__device__ __forceinline__ int tail_start(const int32_t* __restrict__ kl, int first, int n_new) {
+  int lo = first, hi = n_new;
+  while (lo < hi) {
+    const int step = (hi - lo + 7) / 8;
+    int below = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int i = min(lo + j * step, hi - 1);
+      below += __ldg(kl + i) < n_new;
+    }
+    if (below == 0) return lo;
+    // the probes increase (and may repeat hi - 1): the answer lies after the
+    // last one below n_new and not after the next one
+    const int last = min(lo + (below - 1) * step, hi - 1);
+    if (below < 8) hi = min(lo + below * step, hi - 1);
+    lo = last + 1;
+  }
+  return lo;
+}
+
+// Whether the head and tail split applies (not balanced_split): heads of at
+// most a quarter of the moved rows, or too few streams to fill the grid
+// evenly as units.  pre, which holds the prefix sums of the moved rows, then
+// holds those of the tails.  One warp; every CTA of both kernels finds the
+// same.
+__device__ bool head_tail_split(const DevState& st, const Dims& dm, const int32_t* __restrict__ seq_ids,
+                                const int* list, int n_ev, const int32_t* __restrict__ kept, int kept_stride,
+                                int64_t* pre, int lane) {
+  const int64_t total = pre[n_ev];
+  __syncwarp();
+  int64_t acc = 0;
+  for (int base = 0; base < n_ev; base += 32) {
+    const int k = base + lane;
+    int incl = 0;
+    if (k < n_ev) {
+      const int b = list[k], seq = seq_ids[b], n_new = st.n_cache[seq];
+      incl = n_new - tail_start(kept + (size_t)b * kept_stride, st.first_changed[seq], n_new);
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (k < n_ev) pre[k + 1] = acc + incl;
+    acc += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  __syncwarp();
+  return (total - acc) * 4 <= total || (int64_t)n_ev * 2 * dm.L < kUnitRounds * (int64_t)gridDim.x;
+}
+
 // Entry e, stream q (layer * 2 + K|V) and row r (from the entry's first
 // moved slot) of row o of the balanced row space.
 __device__ __forceinline__ void locate_row(const int64_t* pre, int n_ev, int upe, int64_t o, int& e, int& q,
@@ -288,13 +355,18 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   const int n_pairs = kLayers ? n_ev * dm.L : n_ev;
   const int sp = kLayers ? 2 : 2 * dm.L;  // streams per pair
   int64_t pair_rows = 0;
-  bool balanced = false;
+  bool balanced = false, tails = false;   // tails: the balanced rows are the tails, no stash
   if constexpr (kSplit) {
     if (!kLayers) pair_rows = pre[n_ev];
     else if (n_pairs <= kMaxLayerPairs) pair_rows = layer_pairs(st, dm, seq_ids, list, n_ev, pre, lane);
     balanced = (!kLayers || n_pairs <= kMaxLayerPairs) &&
                balanced_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, kLayers, n_pairs, pair_rows * sp,
                               lane);
+    if (!kLayers && !balanced && after_stash &&
+        head_tail_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, pre, lane)) {
+      balanced = tails = true;
+      pair_rows = pre[n_ev];
+    }
   }
 
   // ---- per-stream units only: whole token rows unless too few streams
@@ -377,14 +449,14 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
     c.kvk = a.kvk;
     c.hg = 0;
     const int64_t rest = pre[p + 1] - pre[p] - r;       // rows of the stream from o on
-    c.i = a.first + (int)r;
-    if (o_stop - o < rest) {                             // the chunk ends inside this stream
+    c.i = (tails ? a.n_new - (int)(pre[p + 1] - pre[p]) : a.first) + (int)r;
+    if (!tails && o_stop - o < rest) {                   // the chunk ends inside this stream
       c.end = c.i + (int)(o_stop - o);
       c.stash_at = c.end;
       c.n_new = a.n_new;
       c.row0 = st.stash_row0[blockIdx.x + 1];            // written by compact_stash_kernel (read again after the wait)
     } else {
-      c.end = c.i + (int)rest;
+      c.end = c.i + (int)min(rest, o_stop - o);
       c.stash_at = INT_MAX;
     }
     c.o_end = o + (c.end - c.i);
@@ -552,6 +624,59 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   }
 }
 
+// The heads of the head and tail split, in place: a CTA per (entry, stream,
+// head group) walks its rows in batches, all of a batch's loads before its
+// stores (kept is increasing and kept[i] >= i, so a row's source is not
+// written before its batch).  Rows are cut into pieces of 512 bytes or more
+// until the units fill the grid twice.
+__device__ void move_heads(const DevState& st, const Dims& dm, const KvDev& kv, const int32_t* __restrict__ seq_ids,
+                           const int* list, const int64_t* pre, int n_ev, const int32_t* __restrict__ kept,
+                           int kept_stride) {
+  const int upe = 2 * dm.L, t = threadIdx.x;
+  int hs = 1, vp = dm.H * dm.d / 8;   // pieces per row, 16-byte vectors per piece
+  while ((int64_t)n_ev * upe * hs < 2 * (int64_t)gridDim.x && vp % 2 == 0 && vp / 2 >= 32) {
+    hs *= 2;
+    vp /= 2;
+  }
+  const int rows_max = min(kHeadUnroll * kStashThreads / vp, kMaxHeadRows);
+  const int64_t units = (int64_t)n_ev * upe * hs;
+  __shared__ const char* s_from[2][kMaxHeadRows];
+  __shared__ char* s_to[2][kMaxHeadRows];
+  int par = 0;
+  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+    const int k = (int)(u / (upe * hs)), b = list[k], seq = seq_ids[b];
+    const int q = (int)(u / hs % upe), layer = q >> 1;
+    char* base = (q & 1 ? kv.base[1] : kv.base[0]) + (int64_t)(u % hs) * vp * 16;
+    const int32_t* kl = kept + (size_t)b * kept_stride;
+    const int end = st.n_cache[seq] - (int)(pre[k + 1] - pre[k]);   // the tail's first row
+    for (int i0 = st.first_changed[seq]; i0 < end; i0 += rows_max, par ^= 1) {
+      const int rows = min(rows_max, end - i0);
+      if (t < rows) {
+        const int from = __ldg(kl + i0 + t);
+        const int64_t so = from >= i0 + t ? kv_row_offset(kv, layer, seq, from, dm.T) : -1;
+        const int64_t to = kv_row_offset(kv, layer, seq, i0 + t, dm.T);
+        const bool ok = so >= 0 && to >= 0;
+        if (!ok) set_error(st.err, from < i0 + t ? EPIKV_DEV_KEPT : EPIKV_DEV_SLOT);
+        s_from[par][t] = ok ? base + so * 2 : nullptr;
+        s_to[par][t] = ok ? base + to * 2 : nullptr;
+      }
+      __syncthreads();
+      uint4 v[kHeadUnroll];
+#pragma unroll
+      for (int k = 0; k < kHeadUnroll; ++k) {
+        const int e = t + k * kStashThreads, r = e / vp;
+        if (r < rows && s_from[par][r]) v[k] = __ldcg(reinterpret_cast<const uint4*>(s_from[par][r]) + (e - r * vp));
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < kHeadUnroll; ++k) {
+        const int e = t + k * kStashThreads, r = e / vp;
+        if (r < rows && s_to[par][r]) *(reinterpret_cast<uint4*>(s_to[par][r]) + (e - r * vp)) = v[k];
+      }
+    }
+  }
+}
+
 // Before a balanced compaction: where chunk g begins inside a stream (row a),
 // CTA g saves into stash g the sources of the previous chunk's rows there
 // that lie in [a, n_new) -- the region later chunks overwrite -- row by row
@@ -567,7 +692,7 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
   int64_t* pre = reinterpret_cast<int64_t*>(list + list_ints(n_seq));
   const bool layers = dm.layer_budgets;
   const int sp = layers ? 2 : 2 * dm.L;  // streams per pair
-  __shared__ int s_pairs, s_bal;
+  __shared__ int s_pairs, s_bal, s_heads;
   __shared__ int64_t s_rows;
   if (threadIdx.x < 32) {
     const int n_ev = evicting_entries(st, dm, seq_ids, n_seq, list, layers ? nullptr : pre, threadIdx.x);
@@ -578,7 +703,10 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
     const bool bal = n_ev > 0 && (!layers || n_pairs <= kMaxLayerPairs) &&
                      balanced_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, layers, n_pairs, rows * sp,
                                     threadIdx.x);
+    const bool heads = n_ev > 0 && !layers && !bal &&
+                       head_tail_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, pre, threadIdx.x);
     if (threadIdx.x == 0) {
+      s_heads = heads;
       s_pairs = n_pairs;
       s_rows = rows;
       s_bal = bal;
@@ -586,6 +714,10 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
   }
   __syncthreads();
   const int64_t total = s_rows * sp;
+  if (s_heads) {
+    move_heads(st, dm, kv, seq_ids, list, pre, s_pairs, kept, kept_stride);
+    return;
+  }
   // compact_kernel's CTAs are let in now, or as this kernel ends (kStashEarlyBytes)
   if (total * dm.H * dm.d * 4 <= kStashEarlyBytes) pdl_trigger();
   if (!s_bal || blockIdx.x == 0) return;
