@@ -263,6 +263,41 @@ __device__ __forceinline__ void radix_select(const KeyAt& key_at, int c0, int c1
   if (total_eq) *total_eq = (int)rs.hist[rs.prefix & 255u];  // the last pass's bin: keys equal to theta
 }
 
+// Shared state of select_kernel.
+struct alignas(16) SelectShared {
+  uint32_t hist[4][256];   // one histogram per radix pass, zeroed once
+  int3 pick[4];            // radix_digit's result of each pass
+  int scan[2][32];
+  int first_ev;
+};
+
+// The digit of the rem-th largest of a 256-bin histogram's keys: pick = that
+// digit, its bin's count and how many of the bin are among the rem largest.
+// One warp; lane l owns digits 255 - 8l .. 248 - 8l (two 16-byte loads).
+__device__ __forceinline__ void radix_digit(const uint32_t* hist, int rem, int lane, int3& pick) {
+  const uint4* h4 = reinterpret_cast<const uint4*>(hist) + 2 * (31 - lane);
+  const uint4 hi = h4[1], lo = h4[0];
+  const int c[8] = {(int)hi.w, (int)hi.z, (int)hi.y, (int)hi.x, (int)lo.w, (int)lo.z, (int)lo.y, (int)lo.x};
+  int sum = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) sum += c[j];
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const unsigned hit = __ballot_sync(0xffffffffu, incl >= rem);
+  if (lane == __ffs(hit) - 1) {   // the first lane that reaches the target
+    int before = incl - sum;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (before < rem && before + c[j] >= rem) pick = make_int3(255 - 8 * lane - j, c[j], rem - before);
+      before += c[j];
+    }
+  }
+}
+
 template <bool kChunked>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims dm,
                                                              const int32_t* __restrict__ seq_ids,
@@ -274,13 +309,19 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
   pdl_wait();
   pdl_trigger();
   const int b = blockIdx.x, tid = threadIdx.x;
+  __shared__ SelectShared ss;
+  for (int j = tid; j < 4 * 256; j += kSelThreads) ss.hist[j >> 8][j & 255] = 0u;
+  if (tid == 0) ss.first_ev = INT_MAX;
+  // everything that the decisions need, in two rounds of loads
   const int seq = seq_ids[b];
+  const int K = budget[b];
+  const int trig = trigger ? trigger[b] : K;
   if (seq < 0 || seq >= dm.S) {
     if (tid == 0) set_error(st.err, EPIKV_DEV_BATCH);
     return;
   }
   const int n = st.n_cache[seq];
-  const int K = budget[b];
+  const int prefill = st.prefill[seq], policy = st.policy[seq];
   if (K < 1 || K > dm.T) {
     if (tid == 0) {
       set_error(st.err, EPIKV_DEV_BUDGET);
@@ -289,7 +330,6 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
     }
     return;
   }
-  const int trig = trigger ? trigger[b] : K;
   if (n <= K || n <= trig) {  // nothing to evict
     if (tid == 0) {
       st.first_changed[seq] = n;
@@ -297,7 +337,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
     }
     return;
   }
-  const int P = min(st.prefill[seq], n);
+  const int P = min(prefill, n);
   const int R = min(min(dm.recency_cap, K / 4), max(0, K - P));
   const int M = max(0, K - P - R);
   const int c0 = P, c1 = n - R;  // candidates [c0, c1)
@@ -309,25 +349,9 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
     }
     return;
   }
-  const float* __restrict__ sc = st.score[kind_index(st.policy[seq])] + (size_t)seq * dm.T;
+  const float* __restrict__ sc = st.score[kind_index(policy)] + (size_t)seq * dm.T;
   int32_t* out = kept_out + (size_t)b * kept_stride;
 
-  // ---- chunk keys (chunk-level selection only)
-  uint32_t* __restrict__ ck = kChunked ? st.ckey + (size_t)seq * dm.T : nullptr;
-  if (kChunked) {
-    const int C = dm.select_chunk;
-    const int32_t* __restrict__ pz = st.pos + (size_t)seq * dm.T;
-    for (int i = c0 + tid; i < c1; i += kSelThreads) {
-      const int c = pz[i] / C;
-      if (i > c0 && pz[i - 1] / C == c) continue;  // not the chunk's first candidate
-      float s = 0.f;
-      int j = i;
-      for (; j < c1 && pz[j] / C == c; ++j) s = __fadd_rn(s, sc[j]);  // at most C members
-      const uint32_t k = order_key(__fdiv_rn(s, (float)(j - i)));
-      for (int q = i; q < j; ++q) ck[q] = k;
-    }
-    __syncthreads();
-  }
   // the candidates' keys staged in shared memory when the launch provided room
   // for the cache (every later pass reads them there instead of from L2)
   extern __shared__ uint32_t skey[];
@@ -337,25 +361,50 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
   // from the first candidate on (no slot before it moves): the kept rows are
   // then written from shared memory as the kept list is emitted, with no
   // round trip after the selection.
-  __shared__ uint32_t* s_col[kNumKinds + 1];
-  __shared__ int s_ncol;
-  if (tid == 0) {
-    int q = 0;
-    for (int k = 0; k < kNumKinds; ++k)
-      if (st.score[k]) s_col[q++] = reinterpret_cast<uint32_t*>(st.score[k]) + (size_t)seq * dm.T;
-    s_col[q++] = reinterpret_cast<uint32_t*>(st.pos) + (size_t)seq * dm.T;
-    s_ncol = q;
+  uint32_t* col[kFusedCols];
+  int ncol = 0;
+#pragma unroll
+  for (int c = 0; c < kFusedCols; ++c) col[c] = nullptr;
+#pragma unroll
+  for (int k = 0; k <= kNumKinds; ++k) {
+    uint32_t* p = k < kNumKinds ? reinterpret_cast<uint32_t*>(st.score[k < kNumKinds ? k : 0])
+                                : reinterpret_cast<uint32_t*>(st.pos);
+    if (!p) continue;
+#pragma unroll
+    for (int c = 0; c < kFusedCols; ++c)
+      if (c == ncol) col[c] = p + (size_t)seq * dm.T;
+    ++ncol;
   }
-  __syncthreads();
-  const int ncol = s_ncol;
+  __syncthreads();   // the histograms are zero
   const int kpad = (c1 - c0 + 3) & ~3;
   const bool fused = EPIKV_SEL_FUSED_META && staged && ncol <= kFusedCols &&
                      (int64_t)kpad + (int64_t)(ncol + 1) * n <= smem_words;
   uint32_t* smeta = skey + kpad;  // fused: [ncol][n], column c of slot i at c * n + i
   int* skept = reinterpret_cast<int*>(smeta + (size_t)ncol * n);  // fused: the kept list
-  uint32_t* col[kFusedCols];
-#pragma unroll
-  for (int c = 0; c < kFusedCols; ++c) col[c] = c < ncol ? s_col[c] : nullptr;
+  uint32_t* __restrict__ ck = kChunked ? st.ckey + (size_t)seq * dm.T : nullptr;
+  // ---- chunk keys (chunk-level selection only): the thread owning a chunk's
+  // first candidate sums its scores in slot order
+  auto chunk_keys = [&](const int32_t* pz, const float* ps, auto put) {
+    const int C = dm.select_chunk;
+    for (int i = c0 + tid; i < c1; i += kSelThreads) {
+      const uint32_t lo = (uint32_t)pz[i] / (uint32_t)C * (uint32_t)C;   // the chunk's positions: [lo, lo + C)
+      if (i > c0 && (uint32_t)pz[i - 1] >= lo) continue;  // not the chunk's first candidate
+      float s = 0.f;
+      int j = i;
+      for (; j < c1 && (uint32_t)pz[j] - lo < (uint32_t)C; ++j) s = __fadd_rn(s, ps[j]);  // at most C members
+      const uint32_t k = order_key(__fdiv_rn(s, (float)(j - i)));
+      put(i, j, k);
+    }
+  };
+  // from the staged columns where they are staged: a chunk's members one
+  // after another from L2 took 10 us of the 26 us of a 3,048-slot selection
+  const bool chunk_staged = kChunked && fused;
+  if (kChunked && !fused) {
+    chunk_keys(st.pos + (size_t)seq * dm.T, sc, [&](int i, int j, uint32_t k) {
+      for (int q = i; q < j; ++q) ck[q] = k;
+    });
+    __syncthreads();
+  }
   if (staged) {
     // U slots per thread with every load in flight before the stores
     constexpr int U = 4;
@@ -365,7 +414,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * kSelThreads;
-        if (i < c1) kv[u] = kChunked ? ck[i] : order_key(sc[i]);
+        kv[u] = i < c1 && !chunk_staged ? (kChunked ? ck[i] : order_key(sc[i])) : 0u;
 #pragma unroll
         for (int c = 0; c < kFusedCols; ++c)
           if (fused && c < ncol && i < n) mv[u][c] = __ldcg(col[c] + i);
@@ -373,39 +422,80 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * kSelThreads;
-        if (i < c1) skey[i - c0] = kv[u];
+        if (i < c1 && !chunk_staged) {
+          skey[i - c0] = kv[u];
+          if (M > 0) atomicAdd(&ss.hist[0][kv[u] >> 24], 1u);   // the first radix pass
+        }
 #pragma unroll
         for (int c = 0; c < kFusedCols; ++c)
           if (fused && c < ncol && i < n) smeta[c * n + i] = mv[u][c];
       }
     }
+  }
+  if (chunk_staged) {
     __syncthreads();
+    unsigned on = 0;   // the policy's column: the kinds held before it
+#pragma unroll
+    for (int k = 0; k < kNumKinds; ++k) on |= (st.score[k] != nullptr ? 1u : 0u) << k;
+    const int pc = __popc(on & (unsigned)(policy - 1));
+    chunk_keys(reinterpret_cast<const int32_t*>(smeta) + (ncol - 1) * n, reinterpret_cast<const float*>(smeta) + pc * n,
+               [&](int i, int j, uint32_t k) {
+                 for (int q = i; q < j; ++q) skey[q - c0] = k;
+                 if (M > 0) atomicAdd(&ss.hist[0][k >> 24], (uint32_t)(j - i));
+               });
   }
   auto key_at = [&](int i) -> uint32_t {
     if (staged) return skey[i - c0];
     return kChunked ? ck[i] : order_key(sc[i]);
   };
 
-  __shared__ RadixShared rs;
-  __shared__ int sh_scan[32];
-
-  // ---- radix select of the M-th largest key among the candidates
-  uint32_t theta = 0xFFFFFFFFu;
-  int need_eq = 0, total_eq = 0;  // no key is 0xFFFFFFFF (order_key), so M == 0 keeps no candidate
-  if (M > 0) radix_select(key_at, c0, c1, M, rs, &theta, &need_eq, &total_eq);
+  // ---- radix select of the M-th largest key among the candidates: those with
+  // keys above theta are kept, and those equal to it if all_eq, else the
+  // first need_eq of them by slot.  A pass ends the search when every key
+  // with its leading digits is kept (2 or 3 of 4 passes on most scores).
+  uint32_t theta = 0xFFFFFFFFu;   // no key is 0xFFFFFFFF (order_key), so M == 0 keeps no candidate
+  int need_eq = 0;
+  bool all_eq = true;
+  if (M > 0) {
+    uint32_t prefix = 0u, mask = 0u;
+    int rem = M;
+    for (int pass = 0, shift = 24;; ++pass, shift -= 8) {
+      if (pass > 0 || !staged) {
+        uint32_t* h = ss.hist[pass];
+        for (int i = c0 + tid; i < c1; i += kSelThreads) {
+          const uint32_t k = key_at(i);
+          if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 255u], 1u);
+        }
+      }
+      __syncthreads();
+      if (tid < 32) radix_digit(ss.hist[pass], rem, tid, ss.pick[pass]);
+      __syncthreads();
+      const int3 pk = ss.pick[pass];   // digit, candidates with it, how many of those are kept
+      prefix |= (uint32_t)pk.x << shift;
+      mask |= 255u << shift;
+      rem = pk.z;
+      if (pass == 3 || pk.y == rem) {
+        theta = prefix;   // all_eq: keys from theta on, whatever their later digits
+        need_eq = rem;
+        all_eq = pk.y == rem;
+        break;
+      }
+    }
+  } else {
+    __syncthreads();   // the staged columns
+  }
 
   // ---- ordered scans over contiguous per-thread slot ranges
   const int per = (n + kSelThreads - 1) / kSelThreads;
   const int a = min(n, tid * per), e = min(n, a + per);
   // when every key equal to theta is kept (the usual case), which of them
   // come first does not matter and the count before each thread is not needed
-  const bool all_eq = need_eq == total_eq;
   int eq_base = 0;
   if (!all_eq) {  // uniform across the block
     int eq_local = 0;
     for (int i = max(a, c0); i < min(e, c1); ++i) eq_local += (key_at(i) == theta);
     int tot;
-    eq_base = block_exclusive_scan(eq_local, &tot, sh_scan);
+    eq_base = block_exclusive_scan(eq_local, &tot, ss.scan[0]);
   }
 
   auto kept_slot = [&](int i, int& eqs) -> bool {
@@ -426,32 +516,38 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
       }
     }
   }
+  if (first_ev != INT_MAX) atomicMin(&ss.first_ev, first_ev);
   int n_kept;
-  const int keep_base = block_exclusive_scan(keep_local, &n_kept, sh_scan);
+  const int keep_base = block_exclusive_scan(keep_local, &n_kept, ss.scan[1]);
   {
     int o = keep_base;
     if (per <= 64) {  // uniform across the block
       for (uint64_t m = kmask; m; m &= m - 1) {
         const int i = a + __ffsll((long long)m) - 1;
-        out[o] = i;
-        if (fused) skept[o] = i;
+        if (fused) skept[o] = i;   // to `out` below, coalesced
+        else out[o] = i;
         ++o;
       }
     } else {
       int eqs = eq_base;
       for (int i = a; i < e; ++i)
-        if (kept_slot(i, eqs)) out[o++] = i;
+        if (kept_slot(i, eqs)) {
+          if (fused) skept[o++] = i;
+          else out[o++] = i;
+        }
     }
   }
-  const int fe = min(block_min(first_ev, sh_scan), n_kept);
+  const int fe = min(ss.first_ev, n_kept);
   __syncthreads();  // kept list visible to the whole block
 
   // ---- compact slot metadata in place (kept[i] >= i, increasing i); the
   // staged keys are no longer needed, so their shared memory stages it
   // (fused: every row from the staged columns, coalesced stores)
   if (fused) {
-    for (int o = fe + tid; o < n_kept; o += kSelThreads) {
+    for (int o = tid; o < n_kept; o += kSelThreads) {
       const int i = skept[o];
+      out[o] = i;
+      if (o < fe) continue;
 #pragma unroll
       for (int c = 0; c < kFusedCols; ++c)
         if (c < ncol) col[c][o] = smeta[c * n + i];
