@@ -608,6 +608,60 @@ __global__ void EPIKV_LAG_BOUNDS lagkv_partial_kernel(DevState st, Dims dm, KvDe
   lag_stream<LH, kLagSeg, false, KINDS, SPLIT>(st, dm, kv, seq, t_lo, t_hi, n_new, layer, kvk, nc0);
 }
 
+// A band's statistics over a window of n values of g, newest first (row[0],
+// row[STEP], row[2 * STEP], ...), each a sum in that order by one thread: z of
+// the newest value (Eq. 3; a shifted two-pass, so that a constant window gives
+// exactly 0) and the window's mean (Eq. 2).  The values are taken from shared
+// memory B at a time, so that the sums wait on their own additions and not on
+// a load each (a decode step of 4 sequences 5.6 -> 5.3 us with the early row
+// loads below; in token_kernel, at 48 registers, B = 1 measured best: 242.5
+// us per 64-sequence call, 4 and 8 244 and 246).
+template <int STEP, int B, typename F>
+__device__ __forceinline__ void window_each(const float* row, int n, F&& f) {
+  int k = 0;
+  for (; k + B <= n; k += B) {
+    float v[B];
+#pragma unroll
+    for (int j = 0; j < B; ++j) v[j] = row[(k + j) * STEP];
+#pragma unroll
+    for (int j = 0; j < B; ++j) f(v[j]);
+  }
+  for (; k < n; ++k) f(row[k * STEP]);
+}
+
+template <int STEP, int B = 16>
+__device__ __forceinline__ float window_z(const float* row, int n, float eps) {
+  const float gnew = row[0];
+  float dsum = 0.f;
+  window_each<STEP, B>(row, n, [&](float v) { dsum += v - gnew; });
+  const float mean_d = dsum / (float)n;
+  float dev = 0.f;
+  window_each<STEP, B>(row, n, [&](float v) {
+    const float e = (v - gnew) - mean_d;
+    dev = fmaf(e, e, dev);
+  });
+  const float sigma = sqrtf(dev / (float)n);
+  return -mean_d / (sigma + eps);  // g(t) - mu = -(mean of g - g(t))
+}
+
+template <int STEP, int B = 16>
+__device__ __forceinline__ float window_mean(const float* row, int n) {
+  float sum = 0.f;
+  window_each<STEP, B>(row, n, [&](float v) { sum += v; });
+  return sum / (float)n;
+}
+
+// Takes a ticket: what the CTA wrote before its last barrier is released to,
+// and what the CTAs with earlier tickets released is acquired from, the whole
+// GPU.  One thread; the others follow it through a barrier.  Two
+// __threadfence around a relaxed atomic took 0.6 us longer (a decode step of
+// 4 sequences 5.3 -> 4.7 us).
+__device__ __forceinline__ uint32_t ticket_add(uint32_t* t) {
+  uint32_t old;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(t) : "memory");
+  return old;
+}
+
 #ifndef EPIKV_FIN_TILE
 #define EPIKV_FIN_TILE 16
 #endif
@@ -671,23 +725,11 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
           const int n = min(dm.z_window, pos);
           const float* row = sg + band * span + (pos - pos_base);   // row[-k] = g at position pos - k
           if (dm.kinds & EPIKV_SCORE_BANDZ) {
-            const float gnew = row[0];
-            float dsum = 0.f;
-            for (int k = 0; k < n; ++k) dsum += row[-k] - gnew;
-            const float mean_d = dsum / (float)n;
-            float dev = 0.f;
-            for (int k = 0; k < n; ++k) {
-              const float e = (row[-k] - gnew) - mean_d;
-              dev = fmaf(e, e, dev);
-            }
-            const float sigma = sqrtf(dev / (float)n);
-            const float z = -mean_d / (sigma + dm.z_eps);  // g(t) - mu = -(mean of g - g(t))
+            const float z = window_z<-1>(row, n, dm.z_eps);
             if (band < dm.nA) za = z; else zb = z;
           }
-          if (dm.kinds & EPIKV_SCORE_HSVAR) {  // rolling mean of g (Eq. 2)
-            float sum = 0.f;
-            for (int k = 0; k < n; ++k) sum += row[-k];
-            const float gbar = sum / (float)n;
+          if (dm.kinds & EPIKV_SCORE_HSVAR) {
+            const float gbar = window_mean<-1>(row, n);
             if (band < dm.nA) ma = gbar; else mb = gbar;
           }
         }
@@ -767,10 +809,7 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
   // The last CTA of this sequence commits its counters (no CTA waits).
   __syncthreads();
   if (tid == 0) {
-    __threadfence();
-    const uint32_t done = atomicAdd(&st.ticket[seq], 1u);
-    if (done == gridDim.x - 1) {
-      __threadfence();
+    if (ticket_add(&st.ticket[seq]) == gridDim.x - 1) {
       if (fits) {
         // an eviction selected but not compacted before this update breaks the
         // call order; nothing is left pending for a later compaction either way
@@ -798,36 +837,37 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
 #define EPIKV_TOKEN_MINB 5
 #endif
 
+// A thread's vectors of one band row of D channels, VR = D / 8.
+template <int VPT>
+__device__ __forceinline__ void band_row(const __nv_bfloat16* row, int VR, uint4 (&x)[VPT]) {
+#pragma unroll
+  for (int k = 0; k < VPT; ++k) {
+    const int v = threadIdx.x + k * kGThreads;
+    x[k] = v < VR ? ld_stream16(row + v * 8) : make_uint4(0, 0, 0, 0);
+  }
+}
+
 // One new token's g for one band layer (Eq. 1), from its row and the saved
 // previous row (h_prev), exactly as bandz_g_kernel forms it (same per-thread
 // vectors, fused multiply-adds, warp sums and fixed-order cross-warp sum);
 // the row is saved as the next call's previous row.  Then, for the band
 // kinds' scores (Eq. 3), this band's z of the new g against its window and
-// the window's mean, with score_finalize_kernel's arithmetic and order (the
-// shifted two-pass over g at positions pos, pos-1, ..., pos-n+1, one thread),
-// stored per (sequence, band) for the last CTA to combine.  The window's
-// earlier values are loaded with the rows into `win` (z_window floats of
-// shared memory).  Every thread of a kGThreads block calls it.
-template <int VPT>
-__device__ __forceinline__ void band_token_g(const DevState& st, const Dims& dm, const BandRows& rows,
-                                             int64_t row_stride, int band, int seq, int r0, int pos, int par,
-                                             float* win) {
+// the window's mean, with score_finalize_kernel's arithmetic and order (window_z
+// over g at positions pos, pos-1, ..., pos-n+1, one thread), stored per
+// (sequence, band) for the last CTA to combine.  c and p are the thread's
+// vectors of the row and the previous one (band_row); the window's earlier
+// values are loaded into `win` (z_window floats of shared memory) while those
+// loads are in flight.  Every thread of a kGThreads block calls it.
+template <int VPT, int B>
+__device__ __forceinline__ void band_token_g(const DevState& st, const Dims& dm, const uint4 (&c)[VPT],
+                                             const uint4 (&p)[VPT], int band, int seq, int pos, int par, float* win) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nb = dm.nA + dm.nB;
   const int VR = dm.D >> 3;
   __shared__ float red[kGThreads / 32];
-  const __nv_bfloat16* cur = rows.p[band] + (int64_t)r0 * row_stride;
-  const __nv_bfloat16* prow = st.h_prev + ((size_t)(seq * 2 + par) * nb + band) * dm.D;
   __nv_bfloat16* hp_wr = st.h_prev + ((size_t)(seq * 2 + (par ^ 1)) * nb + band) * dm.D;
   float* ring = st.g_ring + ((size_t)seq * nb + band) * dm.G;
   const int n = pos >= 1 ? min(dm.z_window, pos) : 0;  // the new g's window, itself included
-  uint4 c[VPT], p[VPT];
-#pragma unroll
-  for (int k = 0; k < VPT; ++k) {
-    const int v = tid + k * kGThreads;
-    c[k] = v < VR ? ld_stream16(cur + v * 8) : make_uint4(0, 0, 0, 0);
-    p[k] = v < VR ? ld_stream16(prow + v * 8) : make_uint4(0, 0, 0, 0);
-  }
   for (int k = 1 + tid; k < n; k += kGThreads) win[k] = __ldcg(ring + ((pos - k) & (dm.G - 1)));
   float acc = 0.f;
 #pragma unroll
@@ -859,24 +899,8 @@ __device__ __forceinline__ void band_token_g(const DevState& st, const Dims& dm,
       win[0] = g;
       const float* row = win;  // row[k] = g at position pos - k
       float z = 0.f, gbar = 0.f;
-      if (dm.kinds & EPIKV_SCORE_BANDZ) {
-        const float gnew = row[0];
-        float dsum = 0.f;
-        for (int k = 0; k < n; ++k) dsum += row[k] - gnew;
-        const float mean_d = dsum / (float)n;
-        float dev = 0.f;
-        for (int k = 0; k < n; ++k) {
-          const float e = (row[k] - gnew) - mean_d;
-          dev = fmaf(e, e, dev);
-        }
-        const float sigma = sqrtf(dev / (float)n);
-        z = -mean_d / (sigma + dm.z_eps);
-      }
-      if (dm.kinds & EPIKV_SCORE_HSVAR) {
-        float s = 0.f;
-        for (int k = 0; k < n; ++k) s += row[k];
-        gbar = s / (float)n;
-      }
+      if (dm.kinds & EPIKV_SCORE_BANDZ) z = window_z<1, B>(row, n, dm.z_eps);
+      if (dm.kinds & EPIKV_SCORE_HSVAR) gbar = window_mean<1, B>(row, n);
       st.ztok[(size_t)(seq * 2) * nb + band] = z;
       st.ztok[(size_t)(seq * 2 + 1) * nb + band] = gbar;
     }
@@ -1006,22 +1030,31 @@ __global__ void __launch_bounds__(kGThreads) bandz_token_kernel(DevState st, Dim
   }
   if (n_new == 0) return;
   const int nb = dm.nA + dm.nB;
+  // both of the band's saved rows are loaded with the new one, before the
+  // state says which of them is the previous row (one round trip less; the
+  // step of 4 sequences reads 0.5 MB more from L2)
+  uint4 c[VPT], p[VPT], p1[VPT];
+  const __nv_bfloat16* saved = st.h_prev + ((size_t)(seq * 2) * nb + band) * dm.D;
+  band_row(rows.p[band] + (int64_t)r0 * row_stride, dm.D >> 3, c);
+  band_row(saved, dm.D >> 3, p);
+  band_row(saved + (size_t)nb * dm.D, dm.D >> 3, p1);
   const int nc0 = st.n_cache[seq];
   const int pos = st.n_seen[seq];
+  const int par = st.hp_parity[seq];
   if (nc0 + 1 > dm.T) {
     if (tid == 0 && band == 0) set_error(st.err, EPIKV_DEV_CAPACITY);
     return;
   }
+  if (par) {
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) p[k] = p1[k];
+  }
   __shared__ int s_last;
   extern __shared__ float win[];  // [z_window]: this band's window of g
-  band_token_g<VPT>(st, dm, rows, row_stride, band, seq, r0, pos, st.hp_parity[seq], win);
-  if (tid == 0) {
-    __threadfence();
-    s_last = atomicAdd(&st.ticket[seq], 1u) == (unsigned)(nb - 1);
-  }
+  band_token_g<VPT, 16>(st, dm, c, p, band, seq, pos, par, win);
+  if (tid == 0) s_last = ticket_add(&st.ticket[seq]) == (unsigned)(nb - 1);
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   if (tid < 32) band_token_combine(st, dm, seq, nc0, pos);
   if (tid == 32) token_commit(st, dm, seq, nc0, pos);  // meanwhile: they touch disjoint state
 }
@@ -1061,9 +1094,18 @@ __global__ void __launch_bounds__(kGThreads, EPIKV_TOKEN_MINB) token_kernel(DevS
   extern __shared__ float win[];  // [z_window] (band CTAs): the band's window of g
   if ((int)blockIdx.x < nbc) {
     const int par = st.hp_parity[seq];
-    if (vpt == 1) band_token_g<1>(st, dm, rows, row_stride, blockIdx.x, seq, r0, pos, par, win);
-    else if (vpt == 2) band_token_g<2>(st, dm, rows, row_stride, blockIdx.x, seq, r0, pos, par, win);
-    else band_token_g<4>(st, dm, rows, row_stride, blockIdx.x, seq, r0, pos, par, win);
+    const __nv_bfloat16* cur = rows.p[blockIdx.x] + (int64_t)r0 * row_stride;
+    const __nv_bfloat16* prev = st.h_prev + ((size_t)(seq * 2 + par) * nbc + blockIdx.x) * dm.D;
+    auto go = [&](auto vpt_t) {
+      constexpr int VPT = decltype(vpt_t)::value;
+      uint4 c[VPT], p[VPT];
+      band_row(cur, dm.D >> 3, c);
+      band_row(prev, dm.D >> 3, p);
+      band_token_g<VPT, 1>(st, dm, c, p, blockIdx.x, seq, pos, par, win);
+    };
+    if (vpt == 1) go(std::integral_constant<int, 1>{});
+    else if (vpt == 2) go(std::integral_constant<int, 2>{});
+    else go(std::integral_constant<int, 4>{});
   } else {
     const int sidx = blockIdx.x - nbc;
     const int layer = half ? sidx : sidx >> 1;
@@ -1073,13 +1115,9 @@ __global__ void __launch_bounds__(kGThreads, EPIKV_TOKEN_MINB) token_kernel(DevS
     else lag_stream<LH, 1>(st, dm, kv, seq, 0, 1, 1, layer, sidx & 1, lnc0);
   }
   __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    s_last = atomicAdd(&st.ticket[seq], 1u) == gridDim.x - 1;
-  }
+  if (tid == 0) s_last = ticket_add(&st.ticket[seq]) == gridDim.x - 1;
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   // three warps at once, on disjoint state: the band scores (warp 0), the
   // K/V scores (warp 1) and the commit (warp 2)
   if (nbc && tid < 32) band_token_combine(st, dm, seq, nc0, pos);
