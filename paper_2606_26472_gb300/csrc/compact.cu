@@ -787,18 +787,17 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
 __global__ void compact_consumed_kernel(DevState st, Dims dm, const int32_t* __restrict__ seq_ids, int n_seq) {
   // launched beside the copy, which does not write the lengths: they are
   // loaded before the wait
-  const int b0 = blockIdx.x * blockDim.x + threadIdx.x;
-  const int seq0 = b0 < n_seq ? seq_ids[b0] : -1;
-  const int n0 = seq0 >= 0 && seq0 < dm.S ? st.n_cache[seq0] : 0;
+  const int per = dm.layer_budgets ? dm.L : 1;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, b = i / per, l = i - b * per;
+  const int seq = b < n_seq ? seq_ids[b] : -1;
+  const bool ok = seq >= 0 && seq < dm.S;
+  const int n = ok && l == 0 ? st.n_cache[seq] : 0;
+  const int nl = ok && dm.layer_budgets ? st.n_layer[seq * dm.L + l] : 0;
   pdl_wait();
   pdl_trigger();
-  for (int b = b0; b < n_seq; b += gridDim.x * blockDim.x) {
-    const int seq = b == b0 ? seq0 : seq_ids[b];
-    if (seq < 0 || seq >= dm.S) continue;
-    st.first_changed[seq] = b == b0 ? n0 : st.n_cache[seq];
-    if (dm.layer_budgets)
-      for (int l = 0; l < dm.L; ++l) st.lfirst[seq * dm.L + l] = st.n_layer[seq * dm.L + l];
-  }
+  if (!ok) return;
+  if (l == 0) st.first_changed[seq] = n;
+  if (dm.layer_budgets) st.lfirst[seq * dm.L + l] = nl;
 }
 
 static int g_ctas_per_sm = 0;
@@ -862,7 +861,8 @@ cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const 
   ++*launches;
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  pdl_launch(compact_consumed_kernel, (n_seq + 255) / 256, 256, 0, stream, st, dm, seq_ids, n_seq);
+  const int marks = n_seq * (layers ? dm.L : 1);
+  pdl_launch(compact_consumed_kernel, (marks + 255) / 256, 256, 0, stream, st, dm, seq_ids, n_seq);
   ++*launches;
   return cudaGetLastError();
 }

@@ -198,72 +198,7 @@ constexpr int kFusedCols = 3;
 #define EPIKV_SEL_FUSED_META 1  // 0: the metadata always moved after selecting (compact_metadata)
 #endif
 
-struct RadixShared {
-  uint32_t hist[256];
-  uint32_t prefix, mask, remaining;
-};
-
-// The M-th largest key_at(i) over i in [c0, c1), 0 < M <= c1 - c0, by a
-// 4-pass 8-bit radix select: *theta is that key, *need_eq the number of
-// keys equal to it that belong to the M largest (the lowest slots first) and
-// *total_eq (when given) the number of keys equal to it.
-// Every thread of the block (NT threads) calls it.
-template <int NT = kSelThreads, typename KeyAt>
-__device__ __forceinline__ void radix_select(const KeyAt& key_at, int c0, int c1, int M, RadixShared& rs,
-                                             uint32_t* theta, int* need_eq, int* total_eq = nullptr) {
-  const int tid = threadIdx.x;
-  __syncthreads();  // every thread has read the previous call's result
-  if (tid == 0) {
-    rs.prefix = 0u;
-    rs.mask = 0u;
-    rs.remaining = (uint32_t)M;
-  }
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int j = tid; j < 256; j += NT) rs.hist[j] = 0u;
-    __syncthreads();
-    const uint32_t prefix = rs.prefix, mask = rs.mask;
-    for (int i = c0 + tid; i < c1; i += NT) {
-      const uint32_t k = key_at(i);
-      if ((k & mask) == prefix) atomicAdd(&rs.hist[(k >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (tid < 32) {
-      // lane l owns digits 255-8l .. 248-8l (descending)
-      const int lane = tid;
-      uint32_t lsum = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) lsum += rs.hist[255 - 8 * lane - j];
-      uint32_t incl = lsum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t rem = rs.remaining;
-      const unsigned hit = __ballot_sync(0xffffffffu, incl >= rem);
-      const int owner = __ffs(hit) - 1;  // first lane reaching the target
-      if (lane == owner) {
-        uint32_t before = incl - lsum;
-        for (int j = 0; j < 8; ++j) {
-          const int dg = 255 - 8 * lane - j;
-          if (before + rs.hist[dg] >= rem) {
-            rs.prefix = prefix | ((uint32_t)dg << shift);
-            rs.mask = mask | (255u << shift);
-            rs.remaining = rem - before;
-            break;
-          }
-          before += rs.hist[dg];
-        }
-      }
-    }
-    __syncthreads();
-  }
-  *theta = rs.prefix;
-  *need_eq = (int)rs.remaining;
-  if (total_eq) *total_eq = (int)rs.hist[rs.prefix & 255u];  // the last pass's bin: keys equal to theta
-}
-
-// Shared state of select_kernel.
+// Shared state of the radix searches.
 struct alignas(16) SelectShared {
   uint32_t hist[4][256];   // one histogram per radix pass, zeroed once
   int3 pick[4];            // radix_digit's result of each pass
@@ -800,10 +735,10 @@ __global__ void __cluster_dims__(kCluCtas, 1, 1) __launch_bounds__(kCluThreads)
 
 constexpr int kLayerThreads = 256;
 
-// What both per-layer kernels derive from a sequence's layer budgets.
 // 32-bit words of keep bits per (sequence, layer)
 __host__ __device__ __forceinline__ size_t kKeepWords(int T) { return ((size_t)T + 31) / 32; }
 
+// What both per-layer kernels derive from a sequence's layer budgets.
 struct LayerEvent {
   bool event, bad;
   int n, kmin, kmax, P, R, c0, c1;
@@ -814,15 +749,15 @@ __device__ __forceinline__ LayerEvent layer_event(const DevState& st, const Dims
                                                   const int32_t* __restrict__ trigger) {
   LayerEvent ev;
   ev.n = st.n_cache[seq];
-  ev.kmin = INT_MAX;
-  ev.kmax = 0;
-  ev.bad = false;
-  for (int l = 0; l < dm.L; ++l) {
+  int kmin = INT_MAX, kmax = 0;
+  for (int l = threadIdx.x & 31; l < dm.L; l += 32) {   // a budget per lane
     const int k = budget[(size_t)b * dm.L + l];
-    ev.bad |= k < 1 || k > dm.T;
-    ev.kmin = min(ev.kmin, k);
-    ev.kmax = max(ev.kmax, k);
+    kmin = min(kmin, k);
+    kmax = max(kmax, k);
   }
+  ev.kmin = __reduce_min_sync(0xffffffffu, kmin);
+  ev.kmax = __reduce_max_sync(0xffffffffu, kmax);
+  ev.bad = ev.kmin < 1 || ev.kmax > dm.T;
   const int trig = trigger ? trigger[b] : ev.kmax;
   ev.event = !ev.bad && ev.n > trig && ev.n > ev.kmin;   // some layer is over its budget
   ev.P = min(st.prefill[seq], ev.n);
@@ -869,26 +804,31 @@ __device__ __forceinline__ int warp_base(int v, int* total, int* wt) {
 // candidates), its kept list in its own slot numbering, its new length and
 // first moved slot, and one bit per union slot saying whether the layer
 // keeps it (a 32-bit word per 32 slots, read by layer_union_kernel).
+//
+// Every layer's CTA of a sequence goes over the same scores and masks several
+// times: caches of up to staged_cap slots have the keys, the held bits and the
+// keep bits in shared memory after one pass over them (8 x 32 layers, 6,208
+// slots: 47.6 us reading L2 in every pass, @@KEEP@@ us staged).
 __global__ void __launch_bounds__(kLayerThreads) layer_keep_kernel(DevState st, Dims dm,
                                                                    const int32_t* __restrict__ seq_ids,
                                                                    const int32_t* __restrict__ budget,
                                                                    const int32_t* __restrict__ trigger,
                                                                    int32_t* __restrict__ kept_out, int kept_stride,
-                                                                   int32_t* __restrict__ n_kept_out) {
+                                                                   int32_t* __restrict__ n_kept_out, int staged_cap) {
   pdl_wait();
   pdl_trigger();
   constexpr int NT = kLayerThreads, NW = NT / 32;
   const int l = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, L = dm.L;
   const int lane = tid & 31;
   const unsigned lt = (1u << lane) - 1u;
+  __shared__ SelectShared ss;
+  __shared__ int wt[NW];
+  for (int j = tid; j < 4 * 256; j += NT) ss.hist[j >> 8][j & 255] = 0u;
   const int seq = seq_ids[b];
   if (seq < 0 || seq >= dm.S) {
     if (tid == 0 && l == 0) set_error(st.err, EPIKV_DEV_BATCH);
     return;
   }
-  __shared__ RadixShared rs;
-  __shared__ int sh_scan[32];
-  __shared__ int wt[NW];
   int32_t* nl = st.n_layer + (size_t)seq * L + l;
   int32_t* lf = st.lfirst + (size_t)seq * L + l;
   const LayerEvent ev = layer_event(st, dm, b, seq, budget, trigger);
@@ -907,25 +847,90 @@ __global__ void __launch_bounds__(kLayerThreads) layer_keep_kernel(DevState st, 
   const float* __restrict__ sc = st.score[kind_index(st.policy[seq])] + (size_t)seq * dm.T;
   const unsigned long long* __restrict__ mk = st.lmask + (size_t)seq * dm.T;
   uint32_t* __restrict__ keep = st.lkeep + ((size_t)seq * L + l) * kKeepWords(dm.T);
-  auto key_at = [&](int i) -> uint32_t { return order_key(sc[i]); };
-
-  // threshold of this layer's M best candidates
-  uint32_t theta = 0xFFFFFFFFu;
-  int need_eq = 0;
   const bool all = M >= c1 - c0;  // every candidate passes
   const bool sel = M > 0 && !all;
-  if (sel) radix_select<NT>(key_at, c0, c1, M, rs, &theta, &need_eq);
+
+  extern __shared__ uint32_t lsm[];   // staged: [n] keys, then [words] held bits and [words] keep bits
+  const bool staged = n <= staged_cap;
+  const int words = (n + 31) >> 5;
+  uint32_t* s_held = lsm + n;
+  uint32_t* s_keep = s_held + words;
+  __syncthreads();   // the histograms are zero
+  if (staged) {
+    constexpr int U = 4;   // slots per thread with their loads in flight together
+    for (int i0 = tid - lane; i0 < n; i0 += U * NT) {
+      uint32_t key[U];
+      unsigned long long m[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * NT + lane;
+        m[u] = i < n ? mk[i] : 0ull;
+        key[u] = sel && i >= c0 && i < c1 ? order_key(sc[i]) : 0u;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * NT + lane;
+        const unsigned hb = __ballot_sync(0xffffffffu, (m[u] >> l) & 1ull);
+        if (i < n) lsm[i] = key[u];
+        if (lane == 0 && i < n) s_held[i >> 5] = hb;
+        if (sel && i >= c0 && i < c1) atomicAdd(&ss.hist[0][key[u] >> 24], 1u);
+      }
+    }
+  }
+  auto key_at = [&](int i) -> uint32_t { return staged ? lsm[i] : order_key(sc[i]); };
+  // the held bits of the 32 slots from i0 on (the whole warp calls it)
+  auto held_word = [&](int i0) -> unsigned {
+    if (staged) return s_held[i0 >> 5];
+    const int i = i0 + lane;
+    return __ballot_sync(0xffffffffu, i < n && ((mk[i < n ? i : 0] >> l) & 1ull));
+  };
+
+  // threshold of this layer's M best candidates, as in select_kernel
+  uint32_t theta = 0xFFFFFFFFu;
+  int need_eq = 0;
+  bool all_eq = true;
+  if (sel) {
+    uint32_t prefix = 0u, mask = 0u;
+    int rem = M;
+    for (int pass = 0, shift = 24;; ++pass, shift -= 8) {
+      if (pass > 0 || !staged)
+        for (int i = c0 + tid; i < c1; i += NT) {
+          const uint32_t k = key_at(i);
+          if ((k & mask) == prefix) atomicAdd(&ss.hist[pass][(k >> shift) & 255u], 1u);
+        }
+      __syncthreads();
+      if (tid < 32) radix_digit(ss.hist[pass], rem, tid, ss.pick[pass]);
+      __syncthreads();
+      const int3 pk = ss.pick[pass];
+      prefix |= (uint32_t)pk.x << shift;
+      mask |= 255u << shift;
+      rem = pk.z;
+      if (pass == 3 || pk.y == rem) {
+        theta = prefix;
+        need_eq = rem;
+        all_eq = pk.y == rem;
+        break;
+      }
+    }
+  } else {
+    __syncthreads();
+  }
 
   const WarpSegment sg = warp_segment<NW>(n);
-  // pass 1: per-warp counts of candidates equal to theta and of held slots
+  // pass 1: per-warp counts of held slots and, if not all are kept, of candidates equal to theta
   int ceq = 0, cold = 0;
-  for (int i0 = sg.lo; i0 < sg.hi; i0 += 32) {
-    const int i = i0 + lane;
-    const bool in = i < sg.hi;
-    const bool eq = sel && in && i >= c0 && i < c1 && key_at(i) == theta;
-    const bool held = in && ((mk[i] >> l) & 1ull);
-    ceq += __popc(__ballot_sync(0xffffffffu, eq));
-    cold += __popc(__ballot_sync(0xffffffffu, held));
+  if (staged) {
+    if (sg.lo < sg.hi)   // (an empty segment may start at n, inside the last word)
+      for (int w = (sg.lo >> 5) + lane; w < (sg.hi + 31) >> 5; w += 32) cold += __popc(s_held[w]);
+    cold = __reduce_add_sync(0xffffffffu, cold);
+  }
+  if (!staged || !all_eq) {
+    for (int i0 = sg.lo; i0 < sg.hi; i0 += 32) {
+      const int i = i0 + lane;
+      const bool eq = !all_eq && i < sg.hi && i >= c0 && i < c1 && key_at(i) == theta;
+      ceq += __popc(__ballot_sync(0xffffffffu, eq));
+      if (!staged) cold += __popc(held_word(i0));
+    }
   }
   int n_eq, n_old;
   int q = warp_base<NW>(ceq, &n_eq, wt);
@@ -934,23 +939,28 @@ __global__ void __launch_bounds__(kLayerThreads) layer_keep_kernel(DevState st, 
   int cnew = 0;
   for (int i0 = sg.lo; i0 < sg.hi; i0 += 32) {
     const int i = i0 + lane;
-    const bool in = i < sg.hi;
-    const bool cand = in && i >= c0 && i < c1;
-    const bool held = in && ((mk[i] >> l) & 1ull);
+    const bool cand = i < sg.hi && i >= c0 && i < c1;
+    const unsigned hb = held_word(i0);
+    const bool held = (hb >> lane) & 1u;
     uint32_t key = 0u;
     if (cand && sel) key = key_at(i);
-    const bool eq = cand && sel && key == theta;
-    const unsigned eb = __ballot_sync(0xffffffffu, eq);
-    const int rank = q + __popc(eb & lt);  // among the candidates equal to theta, in slot order
-    q += __popc(eb);
+    bool eq_kept = true;
+    if (!all_eq) {
+      const unsigned eb = __ballot_sync(0xffffffffu, cand && sel && key == theta);
+      eq_kept = q + __popc(eb & lt) < need_eq;   // among the candidates equal to theta, in slot order
+      q += __popc(eb);
+    }
     bool k = held;
     if (cand) {
-      const bool pass = all || (sel && (key > theta || (eq && rank < need_eq)));
+      const bool pass = all || (sel && (key > theta || (key == theta && eq_kept)));
       if (pass && !held) set_error(st.err, EPIKV_DEV_KEPT);  // the layers' caches are not nested
       k = pass && held;
     }
     const unsigned kb = __ballot_sync(0xffffffffu, k);
-    if (lane == 0) keep[i0 >> 5] = kb;  // segments start at multiples of 32
+    if (lane == 0) {   // segments start at multiples of 32
+      keep[i0 >> 5] = kb;
+      if (staged) s_keep[i0 >> 5] = kb;
+    }
     cnew += __popc(kb);
   }
   int n_new;
@@ -959,13 +969,9 @@ __global__ void __launch_bounds__(kLayerThreads) layer_keep_kernel(DevState st, 
   int32_t* out = kept_out + ((size_t)b * L + l) * kept_stride;
   int o = old_base, fe = INT_MAX;
   for (int i0 = sg.lo; i0 < sg.hi; i0 += 32) {
-    const int i = i0 + lane;
-    const bool in = i < sg.hi;
-    const bool held = in && ((mk[i] >> l) & 1ull);
-    const unsigned kb = keep[i0 >> 5];
-    const bool k = (kb >> lane) & 1u;
-    const unsigned hb = __ballot_sync(0xffffffffu, held);
-    if (k) {
+    const unsigned hb = held_word(i0);
+    const unsigned kb = staged ? s_keep[i0 >> 5] : keep[i0 >> 5];
+    if ((kb >> lane) & 1u) {
       const int my_o = o + __popc(hb & lt), my_j = j + __popc(kb & lt);
       if (my_j < kept_stride) out[my_j] = my_o;
       if (my_o != my_j) fe = min(fe, my_j);
@@ -973,7 +979,7 @@ __global__ void __launch_bounds__(kLayerThreads) layer_keep_kernel(DevState st, 
     o += __popc(hb);
     j += __popc(kb);
   }
-  fe = block_min<NT>(fe, sh_scan);
+  fe = block_min<NT>(fe, ss.scan[0]);
   if (tid == 0) {
     if (n_old != *nl) set_error(st.err, EPIKV_DEV_KEPT);  // the masks and the length disagree
     const int f = min(fe, n_new);
@@ -1003,7 +1009,6 @@ __global__ void __launch_bounds__(kSelThreads) layer_union_kernel(DevState st, D
   if (seq < 0 || seq >= dm.S) return;   // reported by layer_keep_kernel
   __shared__ int sh_scan[32];
   __shared__ int wt[NW];
-  __shared__ int s_changed;
   const LayerEvent ev = layer_event(st, dm, b, seq, budget, trigger);
   const int n = ev.n;
   if (!ev.event || max(ev.kmax, ev.P) > kept_stride) {
@@ -1014,25 +1019,35 @@ __global__ void __launch_bounds__(kSelThreads) layer_union_kernel(DevState st, D
   unsigned long long* __restrict__ mn = st.lmask_new + (size_t)seq * dm.T;
   const uint32_t* __restrict__ keep = st.lkeep + (size_t)seq * L * kKeepWords(dm.T);
   const size_t kw = kKeepWords(dm.T);
-  if (tid == 0) {
-    int ch = 0;
-    for (int l = 0; l < L; ++l) ch |= st.lfirst[(size_t)seq * L + l] < st.n_layer[(size_t)seq * L + l];
-    s_changed = ch;
-  }
-  // new masks: a warp takes 32 consecutive slots and one keep word per layer
-  for (int i0 = (tid >> 5) * 32; i0 < n; i0 += kSelThreads) {
-    const int i = i0 + lane;
-    unsigned long long m = 0ull;
-#pragma unroll 8
-    for (int l = 0; l < L; ++l) m |= (unsigned long long)((keep[l * kw + (i0 >> 5)] >> lane) & 1u) << l;
-    if (i < n) mn[i] = m;
-  }
-  __syncthreads();
+  const bool changed = __syncthreads_or(tid < L && st.lfirst[(size_t)seq * L + tid] < st.n_layer[(size_t)seq * L + tid]);
+  // new masks: a warp takes 32 consecutive slots at a time, a lane loads a
+  // layer's keep word (two for more than 32 layers), and the 32 x 32 bits are
+  // exchanged by shuffles; a word per 32 slots, if there is room, for the list
+  extern __shared__ uint32_t stage[];
+  const bool room = (n + 31) >> 5 <= smem_words;
   const WarpSegment sg = warp_segment<NW>(n);
   int cu = 0;
+  uint32_t w0 = 0u, w1 = 0u;
+  auto load_words = [&](int i0) {
+    w0 = i0 < sg.hi && lane < L ? keep[lane * kw + (i0 >> 5)] : 0u;
+    w1 = i0 < sg.hi && lane + 32 < L ? keep[(lane + 32) * kw + (i0 >> 5)] : 0u;
+  };
+  load_words(sg.lo);
   for (int i0 = sg.lo; i0 < sg.hi; i0 += 32) {
     const int i = i0 + lane;
-    cu += __popc(__ballot_sync(0xffffffffu, i < sg.hi && mn[i] != 0ull));
+    const uint32_t c0 = w0, c1 = w1;
+    load_words(i0 + 32);   // the next words, on their way meanwhile
+    uint32_t lo = 0u, hi = 0u;
+#pragma unroll
+    for (int l = 0; l < 32; ++l) lo |= ((__shfl_sync(0xffffffffu, c0, l) >> lane) & 1u) << l;
+    if (L > 32) {
+#pragma unroll
+      for (int l = 0; l < 32; ++l) hi |= ((__shfl_sync(0xffffffffu, c1, l) >> lane) & 1u) << l;
+    }
+    if (i < n) mn[i] = (unsigned long long)hi << 32 | lo;
+    const unsigned kb = __ballot_sync(0xffffffffu, i < sg.hi && (lo | hi) != 0u);
+    if (room && lane == 0) stage[i0 >> 5] = kb;
+    cu += __popc(kb);
   }
   int n_union;
   int o = warp_base<NW>(cu, &n_union, wt);
@@ -1040,9 +1055,8 @@ __global__ void __launch_bounds__(kSelThreads) layer_union_kernel(DevState st, D
   int fe = INT_MAX;
   for (int i0 = sg.lo; i0 < sg.hi; i0 += 32) {
     const int i = i0 + lane;
-    const bool k = i < sg.hi && mn[i] != 0ull;
-    const unsigned kb = __ballot_sync(0xffffffffu, k);
-    if (k) {
+    const unsigned kb = room ? stage[i0 >> 5] : __ballot_sync(0xffffffffu, i < sg.hi && mn[i < n ? i : 0] != 0ull);
+    if ((kb >> lane) & 1u) {
       const int my_o = o + __popc(kb & lt);
       mkept[my_o] = i;
       if (my_o != i) fe = min(fe, my_o);
@@ -1051,13 +1065,12 @@ __global__ void __launch_bounds__(kSelThreads) layer_union_kernel(DevState st, D
   }
   fe = min(block_min(fe, sh_scan), n_union);
   __syncthreads();  // the union's kept list is visible to the whole block
-  extern __shared__ uint32_t stage[];
   compact_metadata(st, dm, seq, mkept, fe, n_union, stage, smem_words);
   // every new mask lands in its slot (the slots before fe did not move)
   for (int j = tid; j < n_union; j += kSelThreads) mk[j] = mn[mkept[j]];
   if (tid == 0) {
     st.n_cache[seq] = n_union;
-    st.first_changed[seq] = s_changed ? 0 : n_union;
+    st.first_changed[seq] = changed ? 0 : n_union;
     atomicAdd(&st.stats[1], 1ull);
     atomicAdd(&st.stats[2], (unsigned long long)(n_union - fe));
   }
@@ -1078,10 +1091,18 @@ static int sel_smem_words(const Dims& dm) {
 }
 static size_t sel_smem(const Dims& dm) { return (size_t)sel_smem_words(dm) * sizeof(uint32_t); }
 
+// layer_keep_kernel's staged slots: 96 KiB of keys at most, so that two CTAs
+// share an SM
+constexpr int kLayerStagedMax = 24 * 1024;
+static size_t layer_smem(int cap) { return cap ? ((size_t)cap + 2 * kKeepWords(cap)) * sizeof(uint32_t) : 0; }
+
 cudaError_t select_prepare() {
   const int mx = kSelStagedMax * (int)sizeof(uint32_t);
   cudaError_t e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(layer_keep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)layer_smem(kLayerStagedMax));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(layer_union_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   return e;
 }
@@ -1093,8 +1114,9 @@ cudaError_t launch_select(const DevState& st, const Dims& dm, int n_seq, const i
   const size_t smem = sel_smem(dm);
   const int words = sel_smem_words(dm);
   if (dm.layer_budgets) {
-    pdl_launch(layer_keep_kernel, dim3(dm.L, n_seq), kLayerThreads, 0, stream, st, dm, seq_ids, budget, trigger,
-               kept, kept_stride, n_kept);
+    const int cap = dm.T <= kLayerStagedMax ? dm.T : 0;
+    pdl_launch(layer_keep_kernel, dim3(dm.L, n_seq), kLayerThreads, layer_smem(cap), stream, st, dm, seq_ids, budget,
+               trigger, kept, kept_stride, n_kept, cap);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     ++*launches;

@@ -38,6 +38,7 @@ def _update(ctx, counts, kv):
     (3, 1, 8, 1, (777, 300), 2, E.EPIKV_LAYOUT_CONTIGUOUS, KV),
     (1, 4, 64, 100, (2400, 1600), 150, E.EPIKV_LAYOUT_PAGED, E.EPIKV_SCORE_LAGKV),
     (1, 4, 64, 16, (900, 640), 17, E.EPIKV_LAYOUT_CONTIGUOUS, E.EPIKV_SCORE_KVKEY | E.EPIKV_SCORE_KVVAL),
+    (32, 1, 32, 16, (600, 533, 600, 257), 3, E.EPIKV_LAYOUT_PAGED, E.EPIKV_SCORE_LAGKV),   # pieces of full length
     (1, 8, 256, 16, (513,), 0, E.EPIKV_LAYOUT_CONTIGUOUS, E.EPIKV_SCORE_LAGKV),
     (2, 8, 128, 600, (1300,), 0, E.EPIKV_LAYOUT_CONTIGUOUS, E.EPIKV_SCORE_LAGKV),   # no cut: pieces shorter than 8 chunks
 ])
