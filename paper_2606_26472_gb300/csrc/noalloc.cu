@@ -47,10 +47,13 @@ constexpr int kTile = 32;
 constexpr int kThreads = 256;
 constexpr int64_t kSms = 152;  // of a GB300
 #ifndef EPIKV_NOALLOC_CTAS
-#define EPIKV_NOALLOC_CTAS 14   // CTAs per SM wanted before pieces get longer: two rounds of 7 resident ones
+#define EPIKV_NOALLOC_CTAS 18   // CTAs per SM wanted before pieces get longer: three rounds of 6 resident ones
 #endif
 #ifndef EPIKV_NOALLOC_CHUNKS
 #define EPIKV_NOALLOC_CHUNKS 2  // shortest piece
+#endif
+#ifndef EPIKV_NOALLOC_PF
+#define EPIKV_NOALLOC_PF 1   // rows prefetched into L2 this many segments ahead (8,192 tokens: 0 237, 1 231, 2 234 us)
 #endif
 #ifndef EPIKV_NOALLOC_MAXREG
 #define EPIKV_NOALLOC_MAXREG 80  // measured best with 72 (128, 80, 72: 171, 128, 127 us on 4,001 tokens; 72 is slower on 200)
@@ -71,8 +74,8 @@ using epikv::KvDev;
 // A piece first takes the minimum and maximum of the chunk before it (bf16
 // values, kept packed; exact), so pieces are independent and one sequence
 // fills the GPU.  A call on 4,001 tokens of a 32-layer cache (524 MB) takes
-// 128 us (4.1 TB/s; bound by its instructions, two passes of arithmetic per
-// row), 200 tokens 19 us; one CTA per stream walking all tokens with a
+// 124 us (4.2 TB/s; bound by its instructions, two passes of arithmetic per
+// row: 75 warp instructions a row, issue active 65 %), 200 tokens 19 us; one CTA per stream walking all tokens with a
 // butterfly per sum took 2,150 and 116 us.  Tokens are taken in segments of up
 // to 8 inside one chunk, their rows loaded together; the variance of a
 // token's head is taken in two passes over the normalised values, four tokens
@@ -104,6 +107,9 @@ __global__ void EPIKV_NOALLOC_BOUNDS noalloc_partial_kernel(KvDev kv, int seq, i
     __syncthreads();
     for (int t = tid; t < gn; t += blockDim.x) soff[t] = kv_row_offset(kv, layer, seq, g0 + t, n);
     __syncthreads();
+    for (int t = tid; t < min(EPIKV_NOALLOC_PF * kSeg, gn); t += blockDim.x)
+      if (soff[t] >= 0)
+        prefetch_l2_bulk((kvk ? kv.base[1] : kv.base[0]) + soff[t] * 2, (uint32_t)(H * d) * 2u);
     for (int i = 0; i < gn;) {
       const int seg = min(min(lag - r, gn - i), kSeg);
       const int t0 = g0 + i;
@@ -114,6 +120,11 @@ __global__ void EPIKV_NOALLOC_BOUNDS noalloc_partial_kernel(KvDev kv, int seq, i
       for (int j = 0; j < kSeg; ++j) {        // past the segment: its last row again, unused sums
         const int64_t off = soff[i + min(j, seg - 1)];
         x[j] = ld_stream16_if(base + off * 2, active && off >= 0);
+      }
+      {   // rows of later segments on their way to L2, each row once
+        const int t = i + EPIKV_NOALLOC_PF * kSeg + tid;
+        if (EPIKV_NOALLOC_PF > 0 && tid < seg && t < gn && soff[t] >= 0)
+          prefetch_l2_bulk((kvk ? kv.base[1] : kv.base[0]) + soff[t] * 2, (uint32_t)(H * d) * 2u);
       }
       if (r == 0) cmn = cmx = x[0];
 #pragma unroll
@@ -221,8 +232,9 @@ __global__ void __launch_bounds__(kThreads) noalloc_finalize_kernel(const float*
 
 // Tokens per piece: as long as there are EPIKV_NOALLOC_CTAS CTAs per SM, since
 // a piece re-reads (from L2) the chunk before it, and at least two chunks
-// (4,001 / 200 tokens: 7 CTAs per SM 141 / 19 us, 14 128 / 19, 28 130 / 19; at
-// least four chunks 130 / 24).
+// (8,192 / 4,001 / 1,000 tokens: 7 CTAs per SM 268 / 141 / 48 us, 12 225 / 123
+// / 44, 14 232 / 127 / 46, 18 222 / 124 / 46, 28 237 / 130 / 46: whole rounds
+// of 6; 200 tokens at least four chunks 24 us, two 19).
 int piece_tokens(int n, int L, int lag) {
   const int64_t least = (int64_t)EPIKV_NOALLOC_CHUNKS * lag, streams = 2 * (int64_t)L;
   const int64_t pieces = (EPIKV_NOALLOC_CTAS * kSms + streams - 1) / streams;
