@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * kSelThreads;
-        kv[u] = i < c1 && !chunk_staged ? (kChunked ? ck[i] : order_key(sc[i])) : 0u;
+        kv[u] = i < c1 && !chunk_staged ? __ldcg(kChunked ? ck + i : reinterpret_cast<const uint32_t*>(sc) + i) : 0u;
 #pragma unroll
         for (int c = 0; c < kFusedCols; ++c)
           if (fused && c < ncol && i < n) mv[u][c] = __ldcg(col[c] + i);
@@ -358,8 +358,9 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
       for (int u = 0; u < U; ++u) {
         const int i = i0 + u * kSelThreads;
         if (i < c1 && !chunk_staged) {
-          skey[i - c0] = kv[u];
-          if (M > 0) atomicAdd(&ss.hist[0][kv[u] >> 24], 1u);   // the first radix pass
+          const uint32_t key = kChunked ? kv[u] : order_key(__uint_as_float(kv[u]));
+          skey[i - c0] = key;
+          if (M > 0) atomicAdd(&ss.hist[0][key >> 24], 1u);   // the first radix pass
         }
 #pragma unroll
         for (int c = 0; c < kFusedCols; ++c)
