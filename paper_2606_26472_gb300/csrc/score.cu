@@ -581,9 +581,21 @@ template <int LH, int KINDS, bool SPLIT>
 __global__ void EPIKV_LAG_BOUNDS lagkv_partial_kernel(DevState st, Dims dm, KvDev kv,
                                                              const int32_t* __restrict__ seq_ids,
                                                              const int32_t* __restrict__ cu_new,
-                                                             int max_new, int piece) {
-  pdl_wait();
+                                                             int max_new, int piece, int beside_g) {
+  // beside_g: launched programmatically after bandz_g_kernel, which lets this
+  // kernel in after its own wait and writes nothing that is read here.  The
+  // two run beside each other (one is bound by its loads, the other by its
+  // instructions: all six kinds of 1,500 and 1,111 tokens 183.5 -> 181.6 us a
+  // call), and every CTA waits before it ends, so that the finalize kernel,
+  // which waits for this one, follows both.
+  if (!beside_g) pdl_wait();
   pdl_trigger();
+  struct WaitAtEnd {
+    bool on;
+    __device__ ~WaitAtEnd() {
+      if (on) pdl_wait();
+    }
+  } at_end{beside_g != 0};
   const int b = blockIdx.y;
   const int seq = seq_ids[b];
   const int n_new = cu_new[b + 1] - cu_new[b];
@@ -662,6 +674,13 @@ __device__ __forceinline__ uint32_t ticket_add(uint32_t* t) {
   return old;
 }
 
+#ifndef EPIKV_FIN_MINB
+// CTAs per SM of the finalize kernel: registers capped at 40 (74 uncapped)
+// for the long calls: 8 prompts of 4,000 tokens at none / 4 / 5 / 6 / 8 CTAs
+// 50 / 39 / 31 / 30 / 27 us, the smallest calls 9.1 / 10.6 / 10.2 / 10.2 /
+// 11.8 us
+#define EPIKV_FIN_MINB 6
+#endif
 #ifndef EPIKV_FIN_TILE
 #define EPIKV_FIN_TILE 16
 #endif
@@ -669,9 +688,10 @@ constexpr int kFinTile = EPIKV_FIN_TILE;  // tokens per finalize CTA
 constexpr int kFinThreads = 256;
 constexpr int kMaxWindow = 1024;
 
-// grid: (token tiles of 32, batch entries); block: 256 threads (warp per token).
+// grid: (token tiles, batch entries, parts: the band kinds, then each K/V kind);
+// block: 256 threads (a warp per token for the K/V kinds).
 template <int WPL>
-__global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st, Dims dm,
+__global__ void __launch_bounds__(kFinThreads, EPIKV_FIN_MINB) score_finalize_kernel(DevState st, Dims dm,
                                                                      const int32_t* __restrict__ seq_ids,
                                                                      const int32_t* __restrict__ cu_new,
                                                                      int max_new) {
@@ -693,24 +713,35 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
   const int i_hi = min(i_lo + kFinTile, n_new);
   const int Gm = dm.G - 1;
   const int nb = dm.nA + dm.nB;
+  // this CTA's part of the kinds: the band kinds first, then one K/V kind each
+  const int part = blockIdx.z, kv_part = (dm.kinds & kBandKinds) ? part - 1 : part;
 
-  extern __shared__ float sg[];  // band kinds: [nb][span] windows of g; then the K/V kinds' u
+  extern __shared__ float sg[];  // band kinds: [nb][span] windows of g; a K/V kind: its u
   if (fits && i_lo < i_hi) {
-    for (int i = i_lo + warp; i < i_hi; i += kFinThreads / 32) {
+    if (part == 0) for (int i = i_lo + warp; i < i_hi; i += kFinThreads / 32) {
       const int pos = p0 + i;
       if (lane == 0) st.pos[(size_t)seq * dm.T + nc0 + i] = pos;
       if (lane == 0 && dm.layer_budgets)  // a new token is in every layer
         st.lmask[(size_t)seq * dm.T + nc0 + i] = dm.L == 64 ? ~0ull : (1ull << dm.L) - 1ull;
     }
-    if (dm.kinds & kBandKinds) {
-      // every g value the tile's windows reach, all band layers, one round of loads
+    if (kv_part < 0) {
+      // every g value the tile's windows reach, all band layers, their loads in flight together
       const int span = kFinTile + dm.z_window - 1;
       const int pos_base = p0 + i_lo - (dm.z_window - 1);  // position held by sg[band][0]
       const int pos_end = p0 + i_hi;
-      for (int idx = tid; idx < nb * span; idx += kFinThreads) {
-        const int band = idx / span;
-        const int pos = pos_base + (idx - band * span);
-        sg[idx] = (pos >= 1 && pos < pos_end) ? st.g_ring[((size_t)seq * nb + band) * dm.G + (pos & Gm)] : 0.f;
+      constexpr int U = 5;   // 15 layers x 79 values: one batch
+      for (int idx0 = tid; idx0 < nb * span; idx0 += U * kFinThreads) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int idx = idx0 + u * kFinThreads, band = idx / span;
+          const int pos = pos_base + (idx - band * span);
+          v[u] = idx < nb * span && pos >= 1 && pos < pos_end
+                     ? __ldcg(st.g_ring + ((size_t)seq * nb + band) * dm.G + (pos & Gm)) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (idx0 + u * kFinThreads < nb * span) sg[idx0 + u * kFinThreads] = v[u];
       }
       __syncthreads();
       // a lane per (token, band layer): lpt lanes per token, 32/lpt tokens per warp
@@ -748,68 +779,57 @@ __global__ void __launch_bounds__(kFinThreads) score_finalize_kernel(DevState st
         }
       }
     }
-    if (dm.kinds & kKvKinds) {
-      // u of the tile's tokens and their windows' earlier ones in this call,
-      // a thread per (kind, token), every kind's loads in flight together and
-      // neighbouring threads' loads side by side (partials [stream][token]):
-      // 4 prompts of 4,099 to 517 tokens 18 us, [token][stream] 23.5 us; all
-      // six kinds of 1,500 and 1,111 tokens 24 us, one kind after another 31 us
-      float* su = sg + (dm.kinds & kBandKinds ? nb * (kFinTile + dm.z_window - 1) : 0);  // [kind][lo .. i_hi)
+    if (kv_part >= 0) {
+      // u of the tile's tokens and their windows' earlier ones in this call, a
+      // thread per token, neighbouring threads' loads side by side (partials
+      // [stream][token])
+      int qk = 0;   // the kv_part-th K/V kind held
+      for (int left = kv_part;; ++qk)
+        if ((dm.kinds & kv_kind(qk)) && left-- == 0) break;
+      const int kind = kv_kind(qk);
+      float* su = sg;  // [lo .. i_hi)
       const int w = dm.lag_window;
       const int lo = max(0, i_lo - (w - 1));
-      const int cnt = i_hi - lo, tile = i_hi - i_lo;
       const float inv_lh = 1.f / (float)(dm.L * dm.H);
-      const int nk = __popc(dm.kinds & kKvKinds);
-      auto nth_kind = [&](int c) -> int {  // the c-th K/V kind held, in kv_kind order
-        int qk = 0;
-        for (int left = c;; ++qk)
-          if ((dm.kinds & kv_kind(qk)) && left-- == 0) return qk;
-      };
-      for (int idx = tid; idx < nk * cnt; idx += kFinThreads) {
-        const int c = idx / cnt, i = lo + (idx - c * cnt);
-        const int kind = kv_kind(nth_kind(c));
-        // which partials: normalised or raw; all (layer, K|V) entries, keys only or values only
-        const bool raw = kind & kRawKinds;
-        const float* pp = (raw ? st.raw_part : st.lag_part) + (size_t)seq * dm.max_new * (2 * dm.L) + i;
-        const int q0 = kind == EPIKV_SCORE_KVVAL ? 1 : 0;
-        const int qs = kind == EPIKV_SCORE_LAGKV ? 1 : 2;
+      // which partials: normalised or raw; all (layer, K|V) entries, keys only or values only
+      const bool raw = kind & kRawKinds;
+      const float* parts = (raw ? st.raw_part : st.lag_part) + (size_t)seq * dm.max_new * (2 * dm.L);
+      const int q0 = kind == EPIKV_SCORE_KVVAL ? 1 : 0;
+      const int qs = kind == EPIKV_SCORE_LAGKV ? 1 : 2;
+      float* ring = st.u_ring[qk] + (size_t)seq * dm.G;
+      float* out = st.score[kind_index(kind)] + (size_t)seq * dm.T + nc0;
+      for (int i = lo + tid; i < i_hi; i += kFinThreads) {
         float u = 0.f;
         if (raw || p0 + i >= dm.lag) {  // the normalised kinds have no value in chunk 0
+          const float* pp = parts + i;
           float s = 0.f;
 #pragma unroll 16
           for (int q = q0; q < 2 * dm.L; q += qs) s += pp[(size_t)q * dm.max_new];
           u = s * inv_lh;
         }
-        su[idx] = u;
+        su[i - lo] = u;
       }
       __syncthreads();
-      for (int it = warp; it < nk * tile; it += kFinThreads / 32) {
-        const int c = it / tile, i = i_lo + (it - c * tile);
-        const int qk = nth_kind(c);
-        const float* ring = st.u_ring[qk] + (size_t)seq * dm.G;
-        const float* us = su + c * cnt - lo;
+      for (int i = i_lo + warp; i < i_hi; i += kFinThreads / 32) {
         const int pos = p0 + i;
         const int n = min(w, pos + 1);
         float acc = 0.f;
 #pragma unroll
         for (int m = 0; m < WPL; ++m) {
           const int k = lane + 32 * m;
-          if (k < n) acc += (i - k >= 0) ? us[i - k] : ring[(pos - k) & Gm];
+          if (k < n) acc += (i - k >= 0) ? su[i - k - lo] : ring[(pos - k) & Gm];
         }
         const float mean = warp_sum(acc) / (float)n;
-        if (lane == 0) st.score[kind_index(kv_kind(qk))][(size_t)seq * dm.T + nc0 + i] = mean;
+        if (lane == 0) out[i] = mean;
       }
-      for (int it = tid; it < nk * tile; it += kFinThreads) {
-        const int c = it / tile, i = i_lo + (it - c * tile);
-        st.u_ring[nth_kind(c)][(size_t)seq * dm.G + ((p0 + i) & Gm)] = su[c * cnt + i - lo];
-      }
+      for (int i = i_lo + tid; i < i_hi; i += kFinThreads) ring[(p0 + i) & Gm] = su[i - lo];
     }
   }
 
   // The last CTA of this sequence commits its counters (no CTA waits).
   __syncthreads();
   if (tid == 0) {
-    if (ticket_add(&st.ticket[seq]) == gridDim.x - 1) {
+    if (ticket_add(&st.ticket[seq]) == gridDim.x * gridDim.z - 1) {
       if (fits) {
         // an eviction selected but not compacted before this update breaks the
         // call order; nothing is left pending for a later compaction either way
@@ -1126,17 +1146,16 @@ __global__ void __launch_bounds__(kGThreads, EPIKV_TOKEN_MINB) token_kernel(DevS
 }
 
 // ------------------------------------------------------------------ launchers
-// dynamic shared memory of the finalize kernel: the band windows of a tile
-// and the K/V kinds' u over it
+// dynamic shared memory of the finalize kernel: the band windows of a tile, or
+// a K/V kind's u over it
 static size_t finalize_smem(const Dims& dm) {
-  size_t words = 0;
-  if (dm.kinds & kBandKinds) words += (size_t)(dm.nA + dm.nB) * (kFinTile + dm.z_window - 1);
-  words += (size_t)__builtin_popcount((unsigned)(dm.kinds & kKvKinds)) * (kFinTile + dm.lag_window - 1);
-  return words * sizeof(float);
+  const size_t band = (dm.kinds & kBandKinds) ? (size_t)(dm.nA + dm.nB) * (kFinTile + dm.z_window - 1) : 0;
+  const size_t kv = (dm.kinds & kKvKinds) ? (size_t)(kFinTile + dm.lag_window - 1) : 0;
+  return (band > kv ? band : kv) * sizeof(float);
 }
 
 cudaError_t finalize_prepare() {
-  const int mx = (int)((size_t)(kMaxBand + 4) * (kFinTile + kMaxWindow - 1) * sizeof(float));
+  const int mx = (int)((size_t)kMaxBand * (kFinTile + kMaxWindow - 1) * sizeof(float));
   const int wmx = (int)((size_t)kMaxBand * kMaxWindow * sizeof(float));
   cudaError_t e = cudaSuccess;
   auto allow = [&](auto kern, int bytes) {
@@ -1257,7 +1276,7 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
     const dim3 grid(2 * dm.L, n_seq, lag_pieces(max_new, dm.lag, piece));
     const int threads = max(32, (dm.H * dm.d / 8 + 31) / 32 * 32);
     auto go = [&](auto kern) {
-      pdl_launch(kern, grid, threads, 0, stream, st, dm, *kv, seq_ids, cu_new, max_new, piece);
+      pdl_launch(kern, grid, threads, 0, stream, st, dm, *kv, seq_ids, cu_new, max_new, piece, band ? 1 : 0);
     };
     auto lanes = [&](auto kinds_t, auto split_t) {
       constexpr int KS = decltype(kinds_t)::value;
@@ -1282,7 +1301,10 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
     ++*launches;
   }
   {
-    const dim3 grid((max_new + kFinTile - 1) / kFinTile, n_seq);
+    // the band kinds and every K/V kind in CTAs of their own: all six kinds of
+    // 1,500 and 1,111 tokens 14 us, one CTA for all of a tile's kinds 24 us
+    const dim3 grid((max_new + kFinTile - 1) / kFinTile, n_seq,
+                    (band ? 1 : 0) + __builtin_popcount((unsigned)(dm.kinds & kKvKinds)));
     const int wmax = max(band ? dm.z_window : 1, (dm.kinds & kKvKinds) ? dm.lag_window : 1);
     const int wpl = (wmax + 31) / 32;
     const size_t smem = finalize_smem(dm);
