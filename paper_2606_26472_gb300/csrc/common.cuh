@@ -63,14 +63,15 @@ struct DevState {
   uint32_t* lkeep;         // [S][L][ceil(T/32)] bit: layer l keeps the union slot (scratch)
   int32_t* mkept;          // [S][T] the select kernel's kept slots of the largest layer (scratch)
   uint32_t* work;          // [2] the compaction's next unit (per-layer budgets) and finished CTAs (0 between launches)
-  char* stash;             // [kMaxStashCtas][stash_rows][H*d] bf16: compaction boundary rows (token budgets)
-  int32_t* stash_row0;     // [kMaxStashCtas] the row whose source is each stash's first row
+  char* stash;             // [kMaxStashCtas][stash_rows][H*d] bf16: compaction boundary rows, fewer per chunk for more chunks
+  int32_t* stash_row0;     // [kMaxChunks] the row whose source is each stash's first row
 };
 
 // The balanced compaction split: at most this many CTAs, each with a stash
 // of at most kStashRows rows (the slots its left neighbour still reads).
 constexpr int kMaxStashCtas = 512;
 constexpr int kStashRows = 128;
+constexpr int kMaxChunks = 1024;   // chunks of a split whose stashes need at most half those rows
 
 struct Dims {
   int S, T, max_new, L, H, d, D, nA, nB, G;

@@ -98,6 +98,61 @@ constexpr int kHeadUnroll = 8;        // vectors per thread and batch of the hea
 constexpr int kMaxHeadRows = 512;     // rows per batch of the head
 constexpr int64_t kUnitRounds = 4;    // streams per CTA from which per-stream units are even enough
 
+// Chunks of the balanced row space: one per CTA, and for long copies more,
+// much shorter ones at its end, which the CTAs take as they finish: some SMs
+// copy more slowly than others, always the same ones (8 x 4,160 contiguous
+// slots in equal chunks: CTAs end between 1,131 and 1,328 us, median 1,195; a
+// paged cache of 32 x 8,320: 9,643 to 9,986, median 9,796).  Each chunk that
+// begins inside a stream needs a stash of `stride` rows, so a stashed split
+// has at most as many chunks as the stash holds, and does this from kLateRows
+// rows per CTA on, where the larger stash pays; the tails of the head and tail
+// split need none.  Equal / late chunks, stash + copy in us:
+//   contiguous (late chunks of 5 % of a CTA's share: 2 %, 3.5 %, 7 % 1,373,
+//   1,298, 1,289): 8 x 4,160 slots 1,356 / 1,275, 20 x 8,100 6,418 / 6,135
+//   paged (2 %, up to 768 chunks): 32 x 8,320 10,118 / 10,028, 8 x 4,160
+//   1,316 / 1,299, 6 x 3,048 in chunks of 16 634 / 613, per-layer budgets
+//   1,314 / 1,309
+//   tails (2 %, eight per CTA): 65,536 + 38,940 + 12,345 to 4,096 slots 461 /
+//   406 (copy), 9,000 to 3,000 97 / 106 (421 rows per CTA: not taken)
+constexpr int kLateRows = 2048, kLateRowsTails = 768;
+constexpr int kChunksPaged = 768;
+constexpr int kLateContiguous = 50, kLatePaged = 20, kLateTails = 20;   // thousandths of a CTA's share
+//
+// kLong: the late chunks are compiled in.  The host takes the other instances
+// for caches too small for them (late_possible): the code alone costs the
+// smallest steps 1.6 us (512 slots 51.9 / 53.5 us, a 2,048-token trace 98.0 /
+// 100.7).
+template <bool kLong>
+struct Chunks {
+  int64_t total, early;   // rows, rows of the first G chunks
+  int G, n;               // CTAs, chunks
+  int stride;             // rows of a chunk's stash
+  __device__ __forceinline__ int64_t start(int c) const {
+    if (!kLong) return total * c / G;
+    return c <= G ? early * c / G : early + (total - early) * (c - G) / (n - G);
+  }
+};
+template <bool kLong>
+__device__ __forceinline__ Chunks<kLong> make_chunks(const Dims& dm, int64_t total, int G, bool tails, int stride,
+                                                     bool paged) {
+  Chunks<kLong> k{total, total, G, G, stride};
+  if (!kLong) return k;
+  int late = 0;
+  if (tails) late = total >= (int64_t)kLateRowsTails * G ? 8 * G : 0;
+  else if (total >= (int64_t)kLateRows * G)
+    late = min(paged ? kChunksPaged : kMaxChunks, kMaxStashCtas * dm.stash_rows / stride) - G;
+  if (late > 0) {
+    k.n = G + late;
+    k.early = total - total * late / G * (tails ? kLateTails : paged ? kLatePaged : kLateContiguous) / 1000;
+  }
+  return k;
+}
+
+// Whether a batch's caches can hold enough rows for late chunks.
+inline bool late_possible(const Dims& dm, int n_seq, int G) {
+  return (int64_t)n_seq * dm.T * 2 * dm.L >= (int64_t)(kLateRows < kLateRowsTails ? kLateRows : kLateRowsTails) * G;
+}
+
 // The balanced split's row space is made of pairs: under token budgets one
 // per evicting entry, with its 2L streams; under per-layer budgets one per
 // (evicting entry, layer), with that layer's K and V streams, at most
@@ -223,20 +278,21 @@ __device__ __forceinline__ PairAt pair_at(const DevState& st, const Dims& dm, co
 // the chunk's last stream segment, no longer than the segment (so than the
 // chunk, ceil(total / grid) rows) nor than the largest shift
 // kept[n-1] - (n-1) of any pair -- within one CTA's stash.  total = moved
-// rows of all streams.
-__device__ bool balanced_split(const DevState& st, const Dims& dm, const int32_t* __restrict__ seq_ids,
+// rows of all streams.  Returns the rows a stash needs, 0 if it does not apply.
+__device__ int balanced_split(const DevState& st, const Dims& dm, const int32_t* __restrict__ seq_ids,
                                const int* list, int n_ev, const int32_t* __restrict__ kept, int kept_stride,
                                bool layers, int n_pairs, int64_t total, int lane) {
-  if (!EPIKV_COMPACT_BALANCED || gridDim.x > kMaxStashCtas) return false;
-  if (layers && n_pairs > kMaxLayerPairs) return false;
-  if ((total + gridDim.x - 1) / gridDim.x <= dm.stash_rows) return true;
-  bool ok = true;
+  if (!EPIKV_COMPACT_BALANCED || gridDim.x > kMaxStashCtas) return 0;
+  if (layers && n_pairs > kMaxLayerPairs) return 0;
+  if ((total + gridDim.x - 1) / gridDim.x <= dm.stash_rows) return dm.stash_rows;
+  int shift = 1;
 #pragma unroll 4
   for (int k = lane; k < n_pairs; k += 32) {
     const PairAt a = pair_at(st, dm, seq_ids, list, kept, kept_stride, layers, k, 0);
-    if (a.n_new > a.first) ok &= __ldg(a.kl + a.n_new - 1) - (a.n_new - 1) <= dm.stash_rows;
+    if (a.n_new > a.first) shift = max(shift, __ldg(a.kl + a.n_new - 1) - (a.n_new - 1));
   }
-  return __all_sync(0xffffffffu, ok);
+  shift = __reduce_max_sync(0xffffffffu, shift);
+  return shift <= dm.stash_rows ? shift : 0;
 }
 
 // The first row in [first, n_new) of a kept list whose source is at or past
@@ -323,7 +379,7 @@ struct Cursor {
 // budgets when the batch has at most kMaxLayerPairs (entry, layer) pairs --
 // the instance for larger batches keeps the per-stream units' code alone,
 // which measured 6 % faster there than with the split's code beside it).
-template <bool kLayers, bool kSplit>
+template <bool kLayers, bool kSplit, bool kLong>
 __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev kv,
                                                      const int32_t* __restrict__ seq_ids, int n_seq,
                                                      const int32_t* __restrict__ kept, int kept_stride,
@@ -355,13 +411,14 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   const int n_pairs = kLayers ? n_ev * dm.L : n_ev;
   const int sp = kLayers ? 2 : 2 * dm.L;  // streams per pair
   int64_t pair_rows = 0;
+  int stride = 0;
   bool balanced = false, tails = false;   // tails: the balanced rows are the tails, no stash
   if constexpr (kSplit) {
     if (!kLayers) pair_rows = pre[n_ev];
     else if (n_pairs <= kMaxLayerPairs) pair_rows = layer_pairs(st, dm, seq_ids, list, n_ev, pre, lane);
-    balanced = (!kLayers || n_pairs <= kMaxLayerPairs) &&
-               balanced_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, kLayers, n_pairs, pair_rows * sp,
-                              lane);
+    if (!kLayers || n_pairs <= kMaxLayerPairs)
+      stride = balanced_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, kLayers, n_pairs, pair_rows * sp, lane);
+    balanced = stride > 0;
     if (!kLayers && !balanced && after_stash &&
         head_tail_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, pre, lane)) {
       balanced = tails = true;
@@ -386,12 +443,14 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   const int rpb = min(kStageBytes / rb, kMaxRPB);      // rows per batch
   const int upe = 2 * dm.L * hs;
   const int units = balanced ? 1 : n_ev * upe;
-  // balanced: this CTA's chunk [o_begin, o_stop) of the row space
+  // balanced: this CTA's current chunk [o_begin, o_stop) of the row space
+  Chunks<kLong> ck{0, 0, G, G, 0};
+  int chunk = blockIdx.x;
   int64_t o_begin = 0, o_stop = 0;
   if (balanced) {
-    const int64_t total = pair_rows * sp;
-    o_begin = (int64_t)blockIdx.x * total / G;
-    o_stop = (int64_t)(blockIdx.x + 1) * total / G;
+    ck = make_chunks<kLong>(dm, pair_rows * sp, G, tails, stride, kv.layout == EPIKV_LAYOUT_PAGED);
+    o_begin = ck.start(chunk);
+    o_stop = ck.start(chunk + 1);
   }
   const bool paged = kv.layout == EPIKV_LAYOUT_PAGED;
   const bool bt_in_smem = paged && kv.max_blocks <= kStagedBlocks;
@@ -454,18 +513,34 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
       c.end = c.i + (int)(o_stop - o);
       c.stash_at = c.end;
       c.n_new = a.n_new;
-      c.row0 = st.stash_row0[blockIdx.x + 1];            // written by compact_stash_kernel (read again after the wait)
+      c.row0 = st.stash_row0[chunk + 1];                 // written by compact_stash_kernel (read again after the wait)
     } else {
       c.end = c.i + (int)min(rest, o_stop - o);
       c.stash_at = INT_MAX;
     }
     c.o_end = o + (c.end - c.i);
   };
+  // balanced: the next late chunk that no CTA has taken (the stash kernel
+  // zeroed the counter)
+  // (-1: none is left)
+  auto next_chunk = [&]() -> int64_t {
+    while (kLong && ck.n > G) {
+      int v = 0;
+      if (lane == 0) v = G + (int)atomicAdd(st.work, 1u);
+      chunk = __shfl_sync(0xffffffffu, v, 0);
+      if (chunk >= ck.n) break;
+      const int64_t o = ck.start(chunk);
+      o_stop = ck.start(chunk + 1);
+      if (o < o_stop) return o;
+    }
+    return -1;
+  };
   auto advance = [&](Cursor& c) {
     c.i += rpb;
     if (c.i >= c.end) {
       if (balanced) {
-        if (c.o_end < o_stop) open_at(c, c.o_end);
+        const int64_t o = c.o_end < o_stop ? c.o_end : next_chunk();
+        if (o >= 0) open_at(c, o);
         else c.u = units;
       } else {
         c.u = next_unit(c.u);
@@ -525,8 +600,8 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
         const char* from_ptr = nullptr;
         if (from >= c.stash_at && from < c.n_new) {  // saved before the copy: a later chunk overwrites it
           const int k = i - c.row0;
-          if (k >= 0 && k < dm.stash_rows)
-            from_ptr = st.stash + ((size_t)(blockIdx.x + 1) * dm.stash_rows + k) * rb;
+          if (k >= 0 && k < ck.stride)
+            from_ptr = st.stash + ((size_t)(chunk + 1) * ck.stride + k) * rb;
         } else if (from >= i) {
           const int64_t so = slot_offset(c.layer, c.seq, from);
           if (so >= 0) from_ptr = kvb + (so + c.hg * piece_elems) * 2;
@@ -569,7 +644,7 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   auto wait_stash = [&] {
     pdl_wait();
     waited = true;
-    if (ld.u < units && ld.stash_at != INT_MAX) ld.row0 = st.stash_row0[blockIdx.x + 1];
+    if (ld.u < units && ld.stash_at != INT_MAX) ld.row0 = st.stash_row0[chunk + 1];
   };
   for (int p = 0; p < kStages - 1 && ld.u < units; ++p) {
     if (!waited) {
@@ -682,11 +757,13 @@ __device__ void move_heads(const DevState& st, const Dims& dm, const KvDev& kv, 
 // that lie in [a, n_new) -- the region later chunks overwrite -- row by row
 // from the first such row (stash_row0[g]).  Nothing of the cache is written,
 // so every read sees the rows as the selection left them.
-__global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState st, Dims dm, KvDev kv,
+template <bool kLong>
+__global__ void __launch_bounds__(kStashThreads, 2) compact_stash_kernel(DevState st, Dims dm, KvDev kv,
                                                                       const int32_t* __restrict__ seq_ids,
                                                                       int n_seq, const int32_t* __restrict__ kept,
                                                                       int kept_stride) {
   pdl_wait();
+  if (kLong && blockIdx.x == 0 && threadIdx.x == 0) st.work[0] = 0u;   // the copy's late chunks
   extern __shared__ __align__(128) unsigned char smem[];
   int* list = reinterpret_cast<int*>(smem);
   int64_t* pre = reinterpret_cast<int64_t*>(list + list_ints(n_seq));
@@ -700,9 +777,10 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
     int64_t rows = 0;
     if (!layers) rows = pre[n_ev];
     else if (n_pairs <= kMaxLayerPairs) rows = layer_pairs(st, dm, seq_ids, list, n_ev, pre, threadIdx.x);
-    const bool bal = n_ev > 0 && (!layers || n_pairs <= kMaxLayerPairs) &&
-                     balanced_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, layers, n_pairs, rows * sp,
-                                    threadIdx.x);
+    const int bal = n_ev > 0 && (!layers || n_pairs <= kMaxLayerPairs)
+                        ? balanced_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, layers, n_pairs, rows * sp,
+                                         threadIdx.x)
+                        : 0;
     const bool heads = n_ev > 0 && !layers && !bal &&
                        head_tail_split(st, dm, seq_ids, list, n_ev, kept, kept_stride, pre, threadIdx.x);
     if (threadIdx.x == 0) {
@@ -720,63 +798,67 @@ __global__ void __launch_bounds__(kStashThreads) compact_stash_kernel(DevState s
   }
   // compact_kernel's CTAs are let in now, or as this kernel ends (kStashEarlyBytes)
   if (total * dm.H * dm.d * 4 <= kStashEarlyBytes) pdl_trigger();
-  if (!s_bal || blockIdx.x == 0) return;
+  if (!s_bal) return;
   const int n_pairs = s_pairs;
-  const int64_t o = (int64_t)blockIdx.x * total / gridDim.x;
-  if (o >= total) return;
-  int p, q;
-  int64_t r;
-  locate_row(pre, n_pairs, sp, o, p, q, r);
-  if (r == 0) return;  // the chunk begins its stream: no other chunk reads its region
-  const PairAt pa = pair_at(st, dm, seq_ids, list, kept, kept_stride, layers, p, q);
-  const int seq = pa.seq, fe = pa.first, n_new = pa.n_new;
-  const int a = fe + (int)r;
-  const int32_t* kl = pa.kl;
-  // the previous chunk's rows in this stream start at seg_start; those whose
-  // sources lie in [a, n_new) are a suffix [i0, i1) of them, at most
-  // stash_rows long (balanced_split), so inside [lo, a)
-  const int64_t s0 = pre[p] * sp + (int64_t)q * (pre[p + 1] - pre[p]);
-  const int64_t o_prev = (int64_t)(blockIdx.x - 1) * total / gridDim.x;
-  const int seg_start = fe + (int)(o_prev > s0 ? o_prev - s0 : 0);
-  const int lo = max(seg_start, a - dm.stash_rows);
-  const int t = threadIdx.x;
+  const Chunks<kLong> ck = make_chunks<kLong>(dm, total, gridDim.x, false, s_bal, kv.layout == EPIKV_LAYOUT_PAGED);
   __shared__ int s_src[kStashRows];  // the sources of rows lo .. a-1
-  const int src = t < a - lo ? __ldg(kl + lo + t) : INT_MAX;
-  if (t < a - lo) s_src[t] = src;
-  const int i0 = lo + __syncthreads_count(src < a);      // kept is increasing: counts of prefixes
-  const int i1 = lo + __syncthreads_count(src < n_new);
-  if (t == 0) st.stash_row0[blockIdx.x] = i0;
-  const int x = i1 - i0;
-  const int layer = pa.layer;
-  const char* kvb = pa.kvk ? kv.base[1] : kv.base[0];
-  const int v16 = dm.H * dm.d / 8;  // 16-byte vectors per row
-  uint4* dst = reinterpret_cast<uint4*>(st.stash + (size_t)blockIdx.x * dm.stash_rows * dm.H * dm.d * 2);
-  // each warp copies two rows at a time, every lane's loads issued before its stores
-  constexpr int kWarps = kStashThreads / 32;
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  for (int r0 = warp; r0 < x; r0 += 2 * kWarps) {
-    const int r1 = r0 + kWarps;
-    const int64_t f0 = kv_row_offset(kv, layer, seq, s_src[i0 - lo + r0], dm.T);
-    const int64_t f1 = r1 < x ? kv_row_offset(kv, layer, seq, s_src[i0 - lo + r1], dm.T) : -2;
-    if ((f0 == -1 || f1 == -1) && lane == 0) set_error(st.err, EPIKV_DEV_SLOT);
-    const uint4* p0 = reinterpret_cast<const uint4*>(kvb + f0 * 2);
-    const uint4* p1 = reinterpret_cast<const uint4*>(kvb + f1 * 2);
-    for (int k0 = lane; k0 < v16; k0 += kStashUnroll * 32) {
-      uint4 v0[kStashUnroll], v1[kStashUnroll];
+  for (int g = blockIdx.x; g < ck.n; g += gridDim.x) {
+    const int64_t o = ck.start(g);
+    if (g == 0 || o >= total) continue;
+    int p, q;
+    int64_t r;
+    locate_row(pre, n_pairs, sp, o, p, q, r);
+    if (r == 0) continue;  // the chunk begins its stream: no other chunk reads its region
+    const PairAt pa = pair_at(st, dm, seq_ids, list, kept, kept_stride, layers, p, q);
+    const int seq = pa.seq, fe = pa.first, n_new = pa.n_new;
+    const int a = fe + (int)r;
+    const int32_t* kl = pa.kl;
+    // the previous chunk's rows in this stream start at seg_start; those whose
+    // sources lie in [a, n_new) are a suffix [i0, i1) of them, at most
+    // stash_rows long (balanced_split), so inside [lo, a)
+    const int64_t s0 = pre[p] * sp + (int64_t)q * (pre[p + 1] - pre[p]);
+    const int64_t o_prev = ck.start(g - 1);
+    const int seg_start = fe + (int)(o_prev > s0 ? o_prev - s0 : 0);
+    const int lo = max(seg_start, a - ck.stride);
+    const int t = threadIdx.x;
+    if (kLong) __syncthreads();  // s_src is reused boundary after boundary
+    const int src = t < a - lo ? __ldg(kl + lo + t) : INT_MAX;
+    if (t < a - lo) s_src[t] = src;
+    const int i0 = lo + __syncthreads_count(src < a);      // kept is increasing: counts of prefixes
+    const int i1 = lo + __syncthreads_count(src < n_new);
+    if (t == 0) st.stash_row0[g] = i0;
+    const int x = i1 - i0;
+    const int layer = pa.layer;
+    const char* kvb = pa.kvk ? kv.base[1] : kv.base[0];
+    const int v16 = dm.H * dm.d / 8;  // 16-byte vectors per row
+    uint4* dst = reinterpret_cast<uint4*>(st.stash + (size_t)g * ck.stride * dm.H * dm.d * 2);
+    // each warp copies two rows at a time, every lane's loads issued before its stores
+    constexpr int kWarps = kStashThreads / 32;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    for (int r0 = warp; r0 < x; r0 += 2 * kWarps) {
+      const int r1 = r0 + kWarps;
+      const int64_t f0 = kv_row_offset(kv, layer, seq, s_src[i0 - lo + r0], dm.T);
+      const int64_t f1 = r1 < x ? kv_row_offset(kv, layer, seq, s_src[i0 - lo + r1], dm.T) : -2;
+      if ((f0 == -1 || f1 == -1) && lane == 0) set_error(st.err, EPIKV_DEV_SLOT);
+      const uint4* p0 = reinterpret_cast<const uint4*>(kvb + f0 * 2);
+      const uint4* p1 = reinterpret_cast<const uint4*>(kvb + f1 * 2);
+      for (int k0 = lane; k0 < v16; k0 += kStashUnroll * 32) {
+        uint4 v0[kStashUnroll], v1[kStashUnroll];
 #pragma unroll
-      for (int u = 0; u < kStashUnroll; ++u) {
-        const int k = k0 + 32 * u;
-        if (k < v16) {
-          if (f0 >= 0) v0[u] = __ldg(p0 + k);
-          if (f1 >= 0) v1[u] = __ldg(p1 + k);
+        for (int u = 0; u < kStashUnroll; ++u) {
+          const int k = k0 + 32 * u;
+          if (k < v16) {
+            if (f0 >= 0) v0[u] = __ldg(p0 + k);
+            if (f1 >= 0) v1[u] = __ldg(p1 + k);
+          }
         }
-      }
 #pragma unroll
-      for (int u = 0; u < kStashUnroll; ++u) {
-        const int k = k0 + 32 * u;
-        if (k < v16) {
-          if (f0 >= 0) dst[(size_t)r0 * v16 + k] = v0[u];
-          if (f1 >= 0) dst[(size_t)r1 * v16 + k] = v1[u];
+        for (int u = 0; u < kStashUnroll; ++u) {
+          const int k = k0 + 32 * u;
+          if (k < v16) {
+            if (f0 >= 0) dst[(size_t)r0 * v16 + k] = v0[u];
+            if (f1 >= 0) dst[(size_t)r1 * v16 + k] = v1[u];
+          }
         }
       }
     }
@@ -817,15 +899,20 @@ cudaError_t compact_prepare(int device, int* ctas_per_sm) {
   auto allow = [&](auto kern) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
   };
-  allow(compact_kernel<false, true>);
-  allow(compact_kernel<true, true>);
-  allow(compact_kernel<true, false>);
+  allow(compact_kernel<false, true, false>);
+  allow(compact_kernel<false, true, true>);
+  allow(compact_kernel<true, true, false>);
+  allow(compact_kernel<true, true, true>);
+  allow(compact_kernel<true, false, false>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(compact_stash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(compact_stash_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)stash_smem(4096, 64, true));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(compact_stash_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)stash_smem(4096, 64, true));
   if (e != cudaSuccess) return e;
   int n = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compact_kernel<false, true>, 32, compact_smem(64, 32, false));
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compact_kernel<false, true, true>, 32, compact_smem(64, 32, false));
   if (e != cudaSuccess) return e;
   g_ctas_per_sm = n > 0 ? n : 1;
   if (EPIKV_COMPACT_CTAS_PER_SM > 0 && EPIKV_COMPACT_CTAS_PER_SM < g_ctas_per_sm)
@@ -842,9 +929,14 @@ cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const 
   const bool split = !layers || n_seq * dm.L <= kMaxLayerPairs;  // the balanced split may apply
   const size_t smem = compact_smem(n_seq, dm.L, layers);
   const bool stash = split && ctas <= kMaxStashCtas;
+  const bool longc = late_possible(dm, n_seq, ctas);
   if (stash) {  // the balanced split's stash (the kernel checks whether it applies)
-    pdl_launch(compact_stash_kernel, ctas, kStashThreads, stash_smem(n_seq, dm.L, layers), stream, st, dm, kv,
-               seq_ids, n_seq, kept, kept_stride);
+    auto go = [&](auto kern) {
+      pdl_launch(kern, ctas, kStashThreads, stash_smem(n_seq, dm.L, layers), stream, st, dm, kv, seq_ids, n_seq, kept,
+                 kept_stride);
+    };
+    if (longc) go(compact_stash_kernel<true>);
+    else go(compact_stash_kernel<false>);
     ++*launches;
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -855,9 +947,9 @@ cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const 
     else
       plain_launch(kern, ctas, 32, smem, stream, st, dm, kv, seq_ids, n_seq, kept, kept_stride, 0);
   };
-  if (!layers) go(compact_kernel<false, true>);
-  else if (split) go(compact_kernel<true, true>);
-  else go(compact_kernel<true, false>);
+  if (!layers) longc ? go(compact_kernel<false, true, true>) : go(compact_kernel<false, true, false>);
+  else if (split) longc ? go(compact_kernel<true, true, true>) : go(compact_kernel<true, true, false>);
+  else go(compact_kernel<true, false, false>);
   ++*launches;
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

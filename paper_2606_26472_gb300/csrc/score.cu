@@ -675,12 +675,14 @@ __device__ __forceinline__ uint32_t ticket_add(uint32_t* t) {
 }
 
 #ifndef EPIKV_FIN_MINB
-// CTAs per SM of the finalize kernel: registers capped at 40 (74 uncapped)
-// for the long calls: 8 prompts of 4,000 tokens at none / 4 / 5 / 6 / 8 CTAs
-// 50 / 39 / 31 / 30 / 27 us, the smallest calls 9.1 / 10.6 / 10.2 / 10.2 /
-// 11.8 us
+// CTAs per SM of the finalize kernel in calls of many tiles: registers capped
+// at 40.  8 prompts of 4,000 tokens at no cap (74) / 4 / 5 / 6 / 8 CTAs 50 /
+// 39 / 31 / 30 / 27 us, 4 prompts of 4,099 to 517 24 / 19 / 16 / 14 / 16.
+// Calls whose tiles are all resident at three CTAs per SM take the instance
+// with the registers for that: a step of 64 new tokens 53.0 -> 49.8 us, 2,048 100.0 -> 94.9.
 #define EPIKV_FIN_MINB 6
 #endif
+constexpr int kFinFree = 3;   // CTAs per SM of the other instance
 #ifndef EPIKV_FIN_TILE
 #define EPIKV_FIN_TILE 16
 #endif
@@ -690,8 +692,8 @@ constexpr int kMaxWindow = 1024;
 
 // grid: (token tiles, batch entries, parts: the band kinds, then each K/V kind);
 // block: 256 threads (a warp per token for the K/V kinds).
-template <int WPL>
-__global__ void __launch_bounds__(kFinThreads, EPIKV_FIN_MINB) score_finalize_kernel(DevState st, Dims dm,
+template <int WPL, bool kMany>
+__global__ void __launch_bounds__(kFinThreads, kMany ? EPIKV_FIN_MINB : kFinFree) score_finalize_kernel(DevState st, Dims dm,
                                                                      const int32_t* __restrict__ seq_ids,
                                                                      const int32_t* __restrict__ cu_new,
                                                                      int max_new) {
@@ -1170,11 +1172,16 @@ cudaError_t finalize_prepare() {
   allow(token_kernel<8>, wmx);
   allow(token_kernel<16>, wmx);
   allow(token_kernel<32>, wmx);
-  allow(score_finalize_kernel<1>, mx);
-  allow(score_finalize_kernel<2>, mx);
-  allow(score_finalize_kernel<4>, mx);
-  allow(score_finalize_kernel<8>, mx);
-  allow(score_finalize_kernel<32>, mx);
+  allow(score_finalize_kernel<1, false>, mx);
+  allow(score_finalize_kernel<2, false>, mx);
+  allow(score_finalize_kernel<4, false>, mx);
+  allow(score_finalize_kernel<8, false>, mx);
+  allow(score_finalize_kernel<32, false>, mx);
+  allow(score_finalize_kernel<1, true>, mx);
+  allow(score_finalize_kernel<2, true>, mx);
+  allow(score_finalize_kernel<4, true>, mx);
+  allow(score_finalize_kernel<8, true>, mx);
+  allow(score_finalize_kernel<32, true>, mx);
   return e;
 }
 
@@ -1309,11 +1316,16 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
     const int wpl = (wmax + 31) / 32;
     const size_t smem = finalize_smem(dm);
     auto go = [&](auto kern) { pdl_launch(kern, grid, kFinThreads, smem, stream, st, dm, seq_ids, cu_new, max_new); };
-    if (wpl <= 1) go(score_finalize_kernel<1>);
-    else if (wpl <= 2) go(score_finalize_kernel<2>);
-    else if (wpl <= 4) go(score_finalize_kernel<4>);
-    else if (wpl <= 8) go(score_finalize_kernel<8>);
-    else go(score_finalize_kernel<32>);
+    auto width = [&](auto many_t) {
+      constexpr bool MANY = decltype(many_t)::value;
+      if (wpl <= 1) go(score_finalize_kernel<1, MANY>);
+      else if (wpl <= 2) go(score_finalize_kernel<2, MANY>);
+      else if (wpl <= 4) go(score_finalize_kernel<4, MANY>);
+      else if (wpl <= 8) go(score_finalize_kernel<8, MANY>);
+      else go(score_finalize_kernel<32, MANY>);
+    };
+    if ((int64_t)grid.x * grid.y * grid.z > (int64_t)kFinFree * num_sms) width(std::true_type{});
+    else width(std::false_type{});
     ++*launches;
   }
   return cudaGetLastError();

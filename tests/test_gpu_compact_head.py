@@ -77,3 +77,17 @@ def test_many_streams_keep_their_units(gpu_lib):
     """24 sequences x 64 streams, 600 -> 300 slots: heads of half the rows and
     five streams per CTA."""
     assert _cut(32, 1, 64, (600,) * 24, (300,) * 24, E.EPIKV_LAYOUT_CONTIGUOUS) == [300] * 24
+
+
+@pytest.mark.parametrize("L,lengths,budgets,layout", [
+    (32, (10200,), (10072,), E.EPIKV_LAYOUT_PAGED),             # shift 128: as many chunks as the whole stash holds
+    (32, (10200,), (10190,), E.EPIKV_LAYOUT_CONTIGUOUS),        # shift 10
+    (64, (5100, 3000, 90, 2500), (5040, 2999, 100, 2440), E.EPIKV_LAYOUT_CONTIGUOUS),
+    (64, (5200, 5150), (5100, 5149), E.EPIKV_LAYOUT_PAGED),
+])
+def test_long_copies_with_late_chunks(gpu_lib, L, lengths, budgets, layout):
+    """More than 2,048 moved rows per CTA: the shorter chunks at the end of the
+    row space, taken as the CTAs finish, and their stashes of the largest
+    shift's rows."""
+    assert _cut(L, 1, 64, lengths, budgets, layout, prefill=(3,) * len(lengths)) == [min(a, b) for a, b in
+                                                                                     zip(lengths, budgets)]
