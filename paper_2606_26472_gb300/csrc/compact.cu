@@ -25,7 +25,8 @@
 // streams come first and the greedy assignment ends nearly level.
 //
 // Balanced split: the moved rows of all evicting streams,
-// laid end to end, are cut into one equal chunk per CTA, so one evicting
+// laid end to end, are cut into one equal chunk per CTA (long copies: and
+// shorter ones for the CTAs that finish first, Chunks below), so one evicting
 // sequence still covers the whole grid and no CTA carries a longer share.
 // A chunk that ends inside a stream at slot a still reads, for its last rows,
 // sources in [a, n_new) that later chunks overwrite.  compact_stash_kernel
@@ -38,8 +39,8 @@
 // from the first one whose source lies at or past the new length, the tail,
 // read slots that no row is written to.  compact_stash_kernel moves the rows
 // before it, the head, in place, a CTA per (stream, head group) in increasing
-// row order; the copy then moves every tail, one equal chunk per CTA, with no
-// row in any chunk's way.  Cutting n slots to K at random leaves about K * K /
+// row order; the copy then moves every tail in chunks, with no row in any
+// chunk's way.  Cutting n slots to K at random leaves about K * K /
 // n rows in the head.  A batch of many streams whose heads are long keeps the
 // per-stream units.  32 layers, 2 KiB rows, units (with their 512-byte to 1
 // KiB pieces) / head + tail: 65,536, 38,940 and 12,345 slots to 4,096 (3.2 GB
@@ -520,8 +521,7 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
     }
     c.o_end = o + (c.end - c.i);
   };
-  // balanced: the next late chunk that no CTA has taken (the stash kernel
-  // zeroed the counter)
+  // balanced: the first row of the next late chunk that no CTA has taken
   // (-1: none is left)
   auto next_chunk = [&]() -> int64_t {
     while (kLong && ck.n > G) {
@@ -763,7 +763,10 @@ __global__ void __launch_bounds__(kStashThreads, 2) compact_stash_kernel(DevStat
                                                                       int n_seq, const int32_t* __restrict__ kept,
                                                                       int kept_stride) {
   pdl_wait();
-  if (kLong && blockIdx.x == 0 && threadIdx.x == 0) st.work[0] = 0u;   // the copy's late chunks
+  // the counter of the copy's late chunks, which the copy first touches after
+  // its wait (under per-layer budgets it may take units before that, and its
+  // last CTA leaves the counter at zero)
+  if (kLong && !dm.layer_budgets && blockIdx.x == 0 && threadIdx.x == 0) st.work[0] = 0u;
   extern __shared__ __align__(128) unsigned char smem[];
   int* list = reinterpret_cast<int*>(smem);
   int64_t* pre = reinterpret_cast<int64_t*>(list + list_ints(n_seq));
