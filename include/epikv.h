@@ -35,8 +35,8 @@
  *     elements (head-major, channel-minor); all pointers 16-byte aligned.
  *   - A sequence id appears at most once in one call's batch.
  *   - A call's kernels are launched with programmatic dependent launch
- *     among themselves (each waits for its predecessor's results before it
- *     reads anything); against the caller's own work on the stream the
+ *     among themselves (each waits for the results that it reads, and ends
+ *     after its predecessor); against the caller's own work on the stream the
  *     order is plain stream order, except that a caller kernel itself
  *     launched with programmatic dependent launch right after a call must,
  *     as with any such launch, wait for its predecessor

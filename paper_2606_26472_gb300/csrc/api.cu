@@ -272,7 +272,7 @@ epikv_status epikv_select(epikv_ctx* ctx, int32_t n_seq, const int32_t* d_seq_id
   int launches = 0;
   ClockScope clock(ctx);
   return cuda_status(launch_select(ctx->st, ctx->dm, n_seq, d_seq_ids, d_budget, d_trigger, d_kept, kept_stride,
-                                   d_n_kept, stream, &launches));
+                                   d_n_kept, false, stream, &launches));
 }
 
 epikv_status epikv_compact(epikv_ctx* ctx, int32_t n_seq, const int32_t* d_seq_ids, const int32_t* d_kept,
@@ -307,7 +307,7 @@ epikv_status epikv_step(epikv_ctx* ctx, int32_t n_seq, const int32_t* d_seq_ids,
   if (ctx->timing) e = cudaEventRecord(ctx->ev[1], stream);
   if (e == cudaSuccess)
     e = launch_select(ctx->st, ctx->dm, n_seq, d_seq_ids, d_budget, d_trigger, ctx->st.kept, ctx->dm.T,
-                      d_n_cache_out ? d_n_cache_out : ctx->st.n_kept, stream, &launches);
+                      d_n_cache_out ? d_n_cache_out : ctx->st.n_kept, max_new > 0, stream, &launches);
   if (e == cudaSuccess && ctx->timing) e = cudaEventRecord(ctx->ev[2], stream);
   if (e == cudaSuccess)
     e = launch_compact(ctx->st, ctx->dm, n_seq, d_seq_ids, ctx->st.kept, ctx->dm.T, kd, ctx->compact_ctas, stream,

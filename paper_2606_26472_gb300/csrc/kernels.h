@@ -11,9 +11,10 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
                                 const int32_t* cu_new, int max_new, const epikv_hidden_view* hv,
                                 const KvDev* kv, int num_sms, cudaStream_t stream, int* launches);
 
+// in_step: launched right after launch_score_update's kernels, in the same call
 cudaError_t launch_select(const DevState& st, const Dims& dm, int n_seq, const int32_t* seq_ids,
                           const int32_t* budget, const int32_t* trigger, int32_t* kept, int kept_stride,
-                          int32_t* n_kept, cudaStream_t stream, int* launches);
+                          int32_t* n_kept, bool in_step, cudaStream_t stream, int* launches);
 
 // Grid of `ctas` persistent CTAs (0: the library's choice for this device).
 cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const int32_t* seq_ids,

@@ -3,7 +3,7 @@
 // One 1024-thread CTA per sequence.  Prefill slots and the trailing recency
 // window R = min(cap, K/4) are always kept; the remaining M = K - P - R slots
 // go to the highest-scoring candidates.  The M-th largest score is found
-// exactly by a 4-pass 8-bit radix select over order-preserving u32 keys
+// exactly by an 8-bit radix select of up to 4 passes over order-preserving u32 keys
 // (NaN lowest, -0 == +0); candidates above the threshold are kept, and of the
 // candidates equal to it the lowest slots are kept.  Two block-wide ordered
 // scans emit the kept list in ascending slot order.  The slot metadata
@@ -240,23 +240,29 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
                                                              const int32_t* __restrict__ trigger,
                                                              int32_t* __restrict__ kept_out, int kept_stride,
                                                              int32_t* __restrict__ n_kept_out, int staged_cap,
-                                                             int smem_words) {
-  pdl_wait();
-  pdl_trigger();
+                                                             int smem_words, int in_step) {
   const int b = blockIdx.x, tid = threadIdx.x;
   __shared__ SelectShared ss;
   for (int j = tid; j < 4 * 256; j += kSelThreads) ss.hist[j >> 8][j & 255] = 0u;
   if (tid == 0) ss.first_ev = INT_MAX;
-  // everything that the decisions need, in two rounds of loads
+  // What the decisions need, in two rounds of loads.  Inside a step (in_step)
+  // the kernel before this one is the call's own score update, which was let
+  // in after the caller's work and writes only the length of what is read
+  // here: all but that is loaded before the wait.
+  if (!in_step) pdl_wait();
   const int seq = seq_ids[b];
   const int K = budget[b];
   const int trig = trigger ? trigger[b] : K;
-  if (seq < 0 || seq >= dm.S) {
+  const bool known = seq >= 0 && seq < dm.S;
+  const int prefill = known ? st.prefill[seq] : 0, policy = known ? st.policy[seq] : 0;
+  __syncthreads();   // the histograms are zero
+  if (in_step) pdl_wait();
+  pdl_trigger();
+  if (!known) {
     if (tid == 0) set_error(st.err, EPIKV_DEV_BATCH);
     return;
   }
   const int n = st.n_cache[seq];
-  const int prefill = st.prefill[seq], policy = st.policy[seq];
   if (K < 1 || K > dm.T) {
     if (tid == 0) {
       set_error(st.err, EPIKV_DEV_BUDGET);
@@ -310,7 +316,6 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(DevState st, Dims d
       if (c == ncol) col[c] = p + (size_t)seq * dm.T;
     ++ncol;
   }
-  __syncthreads();   // the histograms are zero
   const int kpad = (c1 - c0 + 3) & ~3;
   const bool fused = EPIKV_SEL_FUSED_META && staged && ncol <= kFusedCols &&
                      (int64_t)kpad + (int64_t)(ncol + 1) * n <= smem_words;
@@ -1110,7 +1115,7 @@ cudaError_t select_prepare() {
 
 cudaError_t launch_select(const DevState& st, const Dims& dm, int n_seq, const int32_t* seq_ids,
                           const int32_t* budget, const int32_t* trigger, int32_t* kept, int kept_stride,
-                          int32_t* n_kept, cudaStream_t stream, int* launches) {
+                          int32_t* n_kept, bool in_step, cudaStream_t stream, int* launches) {
   if (n_seq == 0) return cudaSuccess;
   const size_t smem = sel_smem(dm);
   const int words = sel_smem_words(dm);
@@ -1125,13 +1130,13 @@ cudaError_t launch_select(const DevState& st, const Dims& dm, int n_seq, const i
                words);
   } else if (dm.select_chunk > 1) {
     pdl_launch(select_kernel<true>, n_seq, kSelThreads, smem, stream, st, dm, seq_ids, budget, trigger, kept,
-               kept_stride, n_kept, sel_staged_cap(dm), words);
+               kept_stride, n_kept, sel_staged_cap(dm), words, in_step ? 1 : 0);
   } else if (dm.T > EPIKV_SEL_CLUSTER_MIN) {
     pdl_launch(select_cluster_kernel, n_seq * kCluCtas, kCluThreads, (size_t)kCluStageWords * sizeof(uint32_t),
                stream, st, dm, seq_ids, budget, trigger, kept, kept_stride, n_kept);
   } else {
     pdl_launch(select_kernel<false>, n_seq, kSelThreads, smem, stream, st, dm, seq_ids, budget, trigger, kept,
-               kept_stride, n_kept, sel_staged_cap(dm), words);
+               kept_stride, n_kept, sel_staged_cap(dm), words, in_step ? 1 : 0);
   }
   ++*launches;
   return cudaGetLastError();
