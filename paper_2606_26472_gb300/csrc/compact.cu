@@ -141,7 +141,8 @@ __device__ __forceinline__ Chunks<kLong> make_chunks(const Dims& dm, int64_t tot
   int late = 0;
   if (tails) late = total >= (int64_t)kLateRowsTails * G ? 8 * G : 0;
   else if (total >= (int64_t)kLateRows * G)
-    late = min(paged ? kChunksPaged : kMaxChunks, kMaxStashCtas * dm.stash_rows / stride) - G;
+    late = min(min(paged ? kChunksPaged : kMaxChunks, kMaxStashCtas * dm.stash_rows / stride) - G,
+               3 * G);   // (of few CTAs: no more than 15 % of the rows)
   if (late > 0) {
     k.n = G + late;
     k.early = total - total * late / G * (tails ? kLateTails : paged ? kLatePaged : kLateContiguous) / 1000;
