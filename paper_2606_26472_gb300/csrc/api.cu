@@ -39,7 +39,7 @@ bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
 bool valid_config(const epikv_config* c) {
   if (!c) return false;
-  if (c->max_seqs < 1 || c->max_seqs > 4096) return false;
+  if (c->max_seqs < 1 || c->max_seqs > kMaxSeqs) return false;
   if (c->max_cache_tokens < 1 || c->max_cache_tokens > (1 << 24)) return false;
   if (c->max_new_tokens < 1 || c->max_new_tokens > (1 << 20)) return false;
   if (c->score_kinds < 1 || c->score_kinds > 63) return false;

@@ -12,6 +12,7 @@
 
 namespace epikv {
 
+constexpr int kMaxSeqs = 4096;  // sequences of a context, so entries of a batch
 constexpr int kMaxBand = 32;
 constexpr int kNumKinds = 6;  // score kind index k <-> mask bit (1 << k)
 constexpr int kBandKinds = EPIKV_SCORE_BANDZ | EPIKV_SCORE_HSVAR;

@@ -898,7 +898,10 @@ static size_t compact_smem(int n_seq, int L, bool layers) {
 
 cudaError_t compact_prepare(int device, int* ctas_per_sm) {
   (void)device;
-  const int mx = (int)compact_smem(4096, 64, true);  // the largest batch and pair table
+  // the largest batch's tables: token budgets take a prefix sum per sequence
+  // (more than the kMaxLayerPairs of per-layer budgets)
+  const int mx = (int)max(compact_smem(kMaxSeqs, 64, false), compact_smem(kMaxSeqs, 64, true));
+  const int mx_stash = (int)max(stash_smem(kMaxSeqs, 64, false), stash_smem(kMaxSeqs, 64, true));
   cudaError_t e = cudaSuccess;
   auto allow = [&](auto kern) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
@@ -909,11 +912,9 @@ cudaError_t compact_prepare(int device, int* ctas_per_sm) {
   allow(compact_kernel<true, true, true>);
   allow(compact_kernel<true, false, false>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(compact_stash_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)stash_smem(4096, 64, true));
+    e = cudaFuncSetAttribute(compact_stash_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx_stash);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(compact_stash_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)stash_smem(4096, 64, true));
+    e = cudaFuncSetAttribute(compact_stash_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx_stash);
   if (e != cudaSuccess) return e;
   int n = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, compact_kernel<false, true, true>, 32, compact_smem(64, 32, false));
