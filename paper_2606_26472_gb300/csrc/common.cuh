@@ -9,6 +9,7 @@
 #include <stdint.h>
 
 #include "epikv.h"
+#include "plans.h"
 
 namespace epikv {
 
@@ -67,12 +68,6 @@ struct DevState {
   char* stash;             // [kMaxStashCtas][stash_rows][H*d] bf16: compaction boundary rows, fewer per chunk for more chunks
   int32_t* stash_row0;     // [kMaxChunks] the row whose source is each stash's first row
 };
-
-// The balanced compaction split: at most this many CTAs, each with a stash
-// of at most kStashRows rows (the slots its left neighbour still reads).
-constexpr int kMaxStashCtas = 512;
-constexpr int kStashRows = 128;
-constexpr int kMaxChunks = 1024;   // chunks of a split whose stashes need at most half those rows
 
 struct Dims {
   int S, T, max_new, L, H, d, D, nA, nB, G;

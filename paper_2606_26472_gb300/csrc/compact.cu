@@ -26,7 +26,7 @@
 //
 // Balanced split: the moved rows of all evicting streams,
 // laid end to end, are cut into one equal chunk per CTA (long copies: and
-// shorter ones for the CTAs that finish first, Chunks below), so one evicting
+// shorter ones for the CTAs that finish first, Chunks in plans.h), so one evicting
 // sequence still covers the whole grid and no CTA carries a longer share.
 // A chunk that ends inside a stream at slot a still reads, for its last rows,
 // sources in [a, n_new) that later chunks overwrite.  compact_stash_kernel
@@ -59,9 +59,6 @@ namespace epikv {
 #ifndef EPIKV_COMPACT_STAGE_BYTES
 #define EPIKV_COMPACT_STAGE_BYTES 16384
 #endif
-#ifndef EPIKV_COMPACT_STAGES
-#define EPIKV_COMPACT_STAGES 4
-#endif
 #ifndef EPIKV_COMPACT_CTAS_PER_SM
 #define EPIKV_COMPACT_CTAS_PER_SM 2  // more CTAs per SM overload the memory system (measured)
 #endif
@@ -72,9 +69,6 @@ namespace epikv {
 #define EPIKV_COMPACT_HEAD_SPLIT 0  // 0: chosen on the device to fill the grid
 #endif
 constexpr int kStageBytes = EPIKV_COMPACT_STAGE_BYTES;
-constexpr int kStages = EPIKV_COMPACT_STAGES;
-constexpr int kMaxRowsPerLane = 4;
-constexpr int kMaxRPB = 32 * kMaxRowsPerLane;
 constexpr uint64_t kWaitNs = 2000000000ull;   // 2 s: far beyond any real copy
 constexpr uint64_t kDrainNs = 100000000ull;   // 0.1 s per stage after a timeout
 
@@ -98,62 +92,6 @@ constexpr int64_t kStashEarlyBytes = 1ll << 30;
 constexpr int kHeadUnroll = 8;        // vectors per thread and batch of the head
 constexpr int kMaxHeadRows = 512;     // rows per batch of the head
 constexpr int64_t kUnitRounds = 4;    // streams per CTA from which per-stream units are even enough
-
-// Chunks of the balanced row space: one per CTA, and for long copies more,
-// much shorter ones at its end, which the CTAs take as they finish: some SMs
-// copy more slowly than others, always the same ones (8 x 4,160 contiguous
-// slots in equal chunks: CTAs end between 1,131 and 1,328 us, median 1,195; a
-// paged cache of 32 x 8,320: 9,643 to 9,986, median 9,796).  Each chunk that
-// begins inside a stream needs a stash of `stride` rows, so a stashed split
-// has at most as many chunks as the stash holds, and does this from kLateRows
-// rows per CTA on, where the larger stash pays; the tails of the head and tail
-// split need none.  Equal / late chunks, stash + copy in us:
-//   contiguous (late chunks of 5 % of a CTA's share: 2 %, 3.5 %, 7 % 1,373,
-//   1,298, 1,289): 8 x 4,160 slots 1,356 / 1,275, 20 x 8,100 6,418 / 6,135
-//   paged (2 %, up to 768 chunks): 32 x 8,320 10,118 / 10,028, 8 x 4,160
-//   1,316 / 1,299, 6 x 3,048 in chunks of 16 634 / 613, per-layer budgets
-//   1,314 / 1,309
-//   tails (2 %, eight per CTA): 65,536 + 38,940 + 12,345 to 4,096 slots 461 /
-//   406 (copy), 9,000 to 3,000 97 / 106 (421 rows per CTA: not taken)
-constexpr int kLateRows = 2048, kLateRowsTails = 768;
-constexpr int kChunksPaged = 768;
-constexpr int kLateContiguous = 50, kLatePaged = 20, kLateTails = 20;   // thousandths of a CTA's share
-//
-// kLong: the late chunks are compiled in.  The host takes the other instances
-// for caches too small for them (late_possible): the code alone costs the
-// smallest steps 1.6 us (512 slots 51.9 / 53.5 us, a 2,048-token trace 98.0 /
-// 100.7).
-template <bool kLong>
-struct Chunks {
-  int64_t total, early;   // rows, rows of the first G chunks
-  int G, n;               // CTAs, chunks
-  int stride;             // rows of a chunk's stash
-  __device__ __forceinline__ int64_t start(int c) const {
-    if (!kLong) return total * c / G;
-    return c <= G ? early * c / G : early + (total - early) * (c - G) / (n - G);
-  }
-};
-template <bool kLong>
-__device__ __forceinline__ Chunks<kLong> make_chunks(const Dims& dm, int64_t total, int G, bool tails, int stride,
-                                                     bool paged) {
-  Chunks<kLong> k{total, total, G, G, stride};
-  if (!kLong) return k;
-  int late = 0;
-  if (tails) late = total >= (int64_t)kLateRowsTails * G ? 8 * G : 0;
-  else if (total >= (int64_t)kLateRows * G)
-    late = min(min(paged ? kChunksPaged : kMaxChunks, kMaxStashCtas * dm.stash_rows / stride) - G,
-               3 * G);   // (of few CTAs: no more than 15 % of the rows)
-  if (late > 0) {
-    k.n = G + late;
-    k.early = total - total * late / G * (tails ? kLateTails : paged ? kLatePaged : kLateContiguous) / 1000;
-  }
-  return k;
-}
-
-// Whether a batch's caches can hold enough rows for late chunks.
-inline bool late_possible(const Dims& dm, int n_seq, int G) {
-  return (int64_t)n_seq * dm.T * 2 * dm.L >= (int64_t)(kLateRows < kLateRowsTails ? kLateRows : kLateRowsTails) * G;
-}
 
 // The balanced split's row space is made of pairs: under token budgets one
 // per evicting entry, with its 2L streams; under per-layer budgets one per
@@ -450,7 +388,7 @@ __global__ void __launch_bounds__(32) compact_kernel(DevState st, Dims dm, KvDev
   int chunk = blockIdx.x;
   int64_t o_begin = 0, o_stop = 0;
   if (balanced) {
-    ck = make_chunks<kLong>(dm, pair_rows * sp, G, tails, stride, kv.layout == EPIKV_LAYOUT_PAGED);
+    ck = make_chunks<kLong>(dm.stash_rows, pair_rows * sp, G, tails, stride, kv.layout == EPIKV_LAYOUT_PAGED);
     o_begin = ck.start(chunk);
     o_stop = ck.start(chunk + 1);
   }
@@ -764,9 +702,9 @@ __global__ void __launch_bounds__(kStashThreads, 2) compact_stash_kernel(DevStat
                                                                       int n_seq, const int32_t* __restrict__ kept,
                                                                       int kept_stride) {
   pdl_wait();
-  // the counter of the copy's late chunks, which the copy first touches after
-  // its wait (under per-layer budgets it may take units before that, and its
-  // last CTA leaves the counter at zero)
+  // the counter of the copy's late chunks, which no CTA of the copy comes to
+  // before its wait (kPrologueRows); under per-layer budgets the copy may take
+  // units before that, and its last CTA leaves the counter at zero
   if (kLong && !dm.layer_budgets && blockIdx.x == 0 && threadIdx.x == 0) st.work[0] = 0u;
   extern __shared__ __align__(128) unsigned char smem[];
   int* list = reinterpret_cast<int*>(smem);
@@ -804,7 +742,7 @@ __global__ void __launch_bounds__(kStashThreads, 2) compact_stash_kernel(DevStat
   if (total * dm.H * dm.d * 4 <= kStashEarlyBytes) pdl_trigger();
   if (!s_bal) return;
   const int n_pairs = s_pairs;
-  const Chunks<kLong> ck = make_chunks<kLong>(dm, total, gridDim.x, false, s_bal, kv.layout == EPIKV_LAYOUT_PAGED);
+  const Chunks<kLong> ck = make_chunks<kLong>(dm.stash_rows, total, gridDim.x, false, s_bal, kv.layout == EPIKV_LAYOUT_PAGED);
   __shared__ int s_src[kStashRows];  // the sources of rows lo .. a-1
   for (int g = blockIdx.x; g < ck.n; g += gridDim.x) {
     const int64_t o = ck.start(g);
@@ -934,7 +872,7 @@ cudaError_t launch_compact(const DevState& st, const Dims& dm, int n_seq, const 
   const bool split = !layers || n_seq * dm.L <= kMaxLayerPairs;  // the balanced split may apply
   const size_t smem = compact_smem(n_seq, dm.L, layers);
   const bool stash = split && ctas <= kMaxStashCtas;
-  const bool longc = late_possible(dm, n_seq, ctas);
+  const bool longc = late_possible(n_seq, dm.T, dm.L, ctas);
   if (stash) {  // the balanced split's stash (the kernel checks whether it applies)
     auto go = [&](auto kern) {
       pdl_launch(kern, ctas, kStashThreads, stash_smem(n_seq, dm.L, layers), stream, st, dm, kv, seq_ids, n_seq, kept,
