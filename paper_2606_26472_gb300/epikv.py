@@ -108,20 +108,29 @@ def _ptr(x):
     return x.data_ptr()
 
 
-_torch_c = None
+_current_stream = None
+
+
+def _current_stream_handle():
+    """What returns torch's current stream as a handle.  torch's own function
+    for that (torch.cuda.current_stream() builds a stream object first, 5 of the
+    18 us that a call of a small step took) is not public: without it, the public
+    one."""
+    import torch
+    torch.cuda.init()
+    raw, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+    if raw is None or device is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
 
 
 def _stream(s):
-    """The CUDA stream handle of a torch stream or an int; None: torch's
-    current stream (asked for as a handle: torch.cuda.current_stream() builds a
-    stream object first, 5 of the 18 us that a call of a small step took)."""
-    global _torch_c
+    """The CUDA stream handle of a torch stream or an int; None: torch's current stream."""
+    global _current_stream
     if s is None:
-        if _torch_c is None:
-            import torch
-            torch.cuda.init()
-            _torch_c = torch._C
-        return _torch_c._cuda_getCurrentRawStream(_torch_c._cuda_getDevice())
+        if _current_stream is None:
+            _current_stream = _current_stream_handle()
+        return _current_stream()
     return s if isinstance(s, int) else s.cuda_stream
 
 
