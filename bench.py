@@ -337,7 +337,8 @@ def stream_bytes(m, *, tokens, seq_calls, rows_moved, kinds, one_token):
     * a token's K and V rows of every layer are read once; with a Lag-KV kind
       each (sequence, call) also reads and writes its range state
       ([L][K|V][4][H][d] bf16);
-    * the compaction reads and writes every moved row."""
+    * the compaction reads and writes every moved row (a deep cut's two moving
+      kernels: deep_cut_bytes)."""
     nb, D = len(m.band_layers), m.hidden
     L, H, d = m.num_layers, m.num_kv_heads, m.head_dim
     band_row = nb * D * 2
@@ -358,6 +359,18 @@ def stream_bytes(m, *, tokens, seq_calls, rows_moved, kinds, one_token):
         if kv:
             out["lagkv_partial_kernel"] = tokens * kv_row + seq_calls * state
     return out
+
+
+def deep_cut_bytes(kept, kv_row):
+    """Algorithmic bytes of a deep cut's two moving kernels, from every
+    sequence's kept list [sequences][K]: compact_stash_kernel itself moves the
+    rows whose source lies below the new length K, compact_kernel those from
+    there on (rows that stay in their slot are not moved)."""
+    K = kept.shape[1]
+    moved = kept != np.arange(K)
+    head = moved & (kept < K)
+    return {"compact_stash_kernel": 2 * int(head.sum()) * kv_row,
+            "compact_kernel": 2 * int((moved & ~head).sum()) * kv_row}
 
 
 def kernel_table(records, n_steps, bytes_per_pass, peak):
@@ -973,12 +986,13 @@ def run_evict64k(args, steps=None, warmup=None):
     s0 = E.epikv_get_stats(ctx)
     recs = kernel_pass(E, ctx, 8, evict)
     s1 = E.epikv_get_stats(ctx)
-    kernels = kernel_table(recs, 1, stream_bytes(m, tokens=0, seq_calls=0, rows_moved=s1["rows_moved"] - s0["rows_moved"],
-                                                 kinds=E.EPIKV_SCORE_BANDZ, one_token=False), peak)
+    row_bytes = L * 2 * H * d * 2
+    kbytes = deep_cut_bytes(kept.cpu().numpy(), row_bytes)
+    assert sum(kbytes.values()) == 2 * (s1["rows_moved"] - s0["rows_moved"]) * row_bytes
+    kernels = kernel_table(recs, 1, kbytes, peak)
     st_, code = E.epikv_get_error(ctx)
     assert st_ == E.EPIKV_OK, f"device error {code}"
     E.epikv_destroy(ctx)
-    row_bytes = L * 2 * H * d * 2
     cbytes = 2 * rows / steps * row_bytes
     c_ms = float(np.median(cmp_))
     return {"workload": "batch4_64k_bandz_single_eviction_to_K4096", "steps": steps, "warmup": warmup,
