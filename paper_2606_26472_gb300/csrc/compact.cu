@@ -224,7 +224,7 @@ __device__ int balanced_split(const DevState& st, const Dims& dm, const int32_t*
                                bool layers, int n_pairs, int64_t total, int lane) {
   if (!EPIKV_COMPACT_BALANCED || gridDim.x > kMaxStashCtas) return 0;
   if (layers && n_pairs > kMaxLayerPairs) return 0;
-  if ((total + gridDim.x - 1) / gridDim.x <= dm.stash_rows) return dm.stash_rows;
+  if (chunks_fit_stash(total, gridDim.x, dm.stash_rows)) return dm.stash_rows;
   int shift = 1;
 #pragma unroll 4
   for (int k = lane; k < n_pairs; k += 32) {
@@ -232,29 +232,7 @@ __device__ int balanced_split(const DevState& st, const Dims& dm, const int32_t*
     if (a.n_new > a.first) shift = max(shift, __ldg(a.kl + a.n_new - 1) - (a.n_new - 1));
   }
   shift = __reduce_max_sync(0xffffffffu, shift);
-  return shift <= dm.stash_rows ? shift : 0;
-}
-
-// The first row in [first, n_new) of a kept list whose source is at or past
-// n_new (n_new if none): an eight-way search, its probes loaded together.
-__device__ __forceinline__ int tail_start(const int32_t* __restrict__ kl, int first, int n_new) {
-  int lo = first, hi = n_new;
-  while (lo < hi) {
-    const int step = (hi - lo + 7) / 8;
-    int below = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int i = min(lo + j * step, hi - 1);
-      below += __ldg(kl + i) < n_new;
-    }
-    if (below == 0) return lo;
-    // the probes increase (and may repeat hi - 1): the answer lies after the
-    // last one below n_new and not after the next one
-    const int last = min(lo + (below - 1) * step, hi - 1);
-    if (below < 8) hi = min(lo + below * step, hi - 1);
-    lo = last + 1;
-  }
-  return lo;
+  return shift_stride(shift, dm.stash_rows);
 }
 
 // Whether the head and tail split applies (not balanced_split): heads of at
@@ -273,7 +251,8 @@ __device__ bool head_tail_split(const DevState& st, const Dims& dm, const int32_
     int incl = 0;
     if (k < n_ev) {
       const int b = list[k], seq = seq_ids[b], n_new = st.n_cache[seq];
-      incl = n_new - tail_start(kept + (size_t)b * kept_stride, st.first_changed[seq], n_new);
+      const int32_t* kl = kept + (size_t)b * kept_stride;
+      incl = n_new - tail_start([kl](int i) { return __ldg(kl + i); }, st.first_changed[seq], n_new);
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

@@ -1,6 +1,7 @@
-// The arithmetic of the compaction's chunks: how the copy kernel cuts its row
-// space.  Plain C++ as well as device code, so that the plans that the
-// kernels follow can be checked on the host as they stand here.
+// The arithmetic of the split kernels' plans: the chunks of the compaction's row
+// space, the head and tail of a deep cut, the pieces of a long K/V score
+// update.  Plain C++ as well as device code, so that the plans that the kernels
+// follow can be checked on the host as they stand here.
 #pragma once
 
 #include <stdint.h>
@@ -25,6 +26,11 @@ constexpr int kMaxChunks = 1024;   // chunks of a split whose stashes need at mo
 constexpr int kStages = EPIKV_COMPACT_STAGES;   // batches of rows that a CTA of the copy has in flight
 constexpr int kMaxRowsPerLane = 4;
 constexpr int kMaxRPB = 32 * kMaxRowsPerLane;   // rows per batch, at most
+
+// Rows of a chunk's stash, 0 if the balanced split does not apply: any chunk's
+// own rows if none is longer than the stash, else the evictions' largest shift.
+EPIKV_PLAN bool chunks_fit_stash(int64_t total, int G, int stash_rows) { return (total + G - 1) / G <= stash_rows; }
+EPIKV_PLAN int shift_stride(int shift, int stash_rows) { return shift <= stash_rows ? shift : 0; }
 
 // Chunks of the balanced row space: one per CTA, and for long copies more,
 // much shorter ones at its end, which the CTAs take as they finish: some SMs
@@ -100,6 +106,75 @@ EPIKV_PLAN Chunks<kLong> make_chunks(int stash_rows, int64_t total, int G, bool 
 // enough rows for late chunks.
 inline bool late_possible(int n_seq, int slots, int L, int G) {
   return (int64_t)n_seq * slots * 2 * L >= (int64_t)(kLateRows < kLateRowsTails ? kLateRows : kLateRowsTails) * G;
+}
+
+// The first row in [first, n_new) of a kept list (at(i): its i-th slot) whose
+// source is at or past n_new (n_new if none): an eight-way search, its probes
+// loaded together.
+template <typename At>
+EPIKV_PLAN int tail_start(const At& at, int first, int n_new) {
+  int lo = first, hi = n_new;
+  while (lo < hi) {
+    const int step = (hi - lo + 7) / 8;
+    int below = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int i = lo + j * step < hi - 1 ? lo + j * step : hi - 1;
+      below += at(i) < n_new;
+    }
+    if (below == 0) return lo;
+    // the probes increase (and may repeat hi - 1): the answer lies after the
+    // last one below n_new and not after the next one
+    const int last = lo + (below - 1) * step < hi - 1 ? lo + (below - 1) * step : hi - 1;
+    if (below < 8) hi = lo + below * step < hi - 1 ? lo + below * step : hi - 1;
+    lo = last + 1;
+  }
+  return lo;
+}
+
+// Piece z of a K/V score update of n_new tokens starting at position p0, in
+// pieces of `piece` tokens (a multiple of lag, at least 4 * lag; 0: one piece):
+// the cuts lie at chunk boundaries, the first piece is two chunks shorter (it
+// reads up to that much at the end of the call for the state), and the rows
+// of the chunk before every cut belong to the call.
+EPIKV_PLAN int lag_piece_start(int p0, int lag, int piece, int z) {
+  return z == 0 ? 0 : (lag - p0 % lag) % lag + z * piece - 2 * lag;
+}
+// pieces that cover max_new tokens from any position
+inline int lag_pieces(int max_new, int lag, int piece) {
+  return piece ? (max_new + 2 * lag + piece - 1) / piece : 1;
+}
+
+#ifndef EPIKV_LAG_PIECE
+#define EPIKV_LAG_PIECE 128  // shortest piece (tokens); never under 8 chunks, nor 4 in small calls
+#endif
+#ifndef EPIKV_LAG_CTAS
+#define EPIKV_LAG_CTAS 56    // CTAs per SM wanted before pieces get longer: 8 rounds of 7 resident ones
+#endif
+// Tokens per piece of the K/V scoring kernel (lag_piece_start), 0 for one
+// piece per stream.  One CTA per (layer, K|V, sequence) leaves a call of few
+// sequences at one or two CTAs per SM, each a serial chain of loads: 4
+// prompts of 4,099 to 517 tokens, 32 layers, took 695 us (1.7 TB/s), all six
+// kinds of 2 prompts of 1,500 and 1,111 tokens 502 us.  Cut into pieces:
+// 231 us (5.2 TB/s) and 125 us.  A piece re-reads the chunk before it (L2),
+// so it has at least 8 chunks; 128 against 256 tokens 125 / 139 us on the
+// second call, and 7, 14, 28, 100 CTAs per SM 274, 247, 234, 224 us on the
+// first.  A call of less than two pieces stays whole (128 tokens of 32
+// sequences fill the GPU as they are).
+inline int lag_piece_tokens(int L, int lag_tokens, int n_seq, int max_new, int num_sms) {
+  const int64_t lag = lag_tokens, streams = (int64_t)2 * L * n_seq;
+  // half as long where whole pieces would not even fill one round of 7 CTAs
+  // per SM: one prompt of 700 tokens 35 -> 29 us
+  const bool few = streams * max_new < (int64_t)7 * num_sms * EPIKV_LAG_PIECE;
+  const int64_t shortest = EPIKV_LAG_PIECE >> few, chunks = 8 >> few;
+  const int64_t least = (shortest > chunks * lag ? (shortest + lag - 1) / lag * lag : chunks * lag);
+  if (max_new < 2 * least) return 0;
+  const int64_t want = (int64_t)EPIKV_LAG_CTAS * num_sms;
+  const int64_t pieces = (want + streams - 1) / streams;
+  int64_t piece = (max_new + pieces - 1) / pieces;
+  piece = (piece + lag - 1) / lag * lag;
+  if (piece < least) piece = least;
+  return piece < max_new ? (int)piece : 0;
 }
 
 }  // namespace epikv

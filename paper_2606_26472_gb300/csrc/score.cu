@@ -250,7 +250,7 @@ __device__ __forceinline__ void lag_moments(const uint4& x, const f32x2 (&a)[4],
 //
 // The stream's tokens [t_lo, t_hi) of the call's n_new are taken: all of them,
 // or (SPLIT) one piece of a long call, cut at chunk boundaries by
-// lag_piece so that few sequences still fill the GPU.  A later piece forms
+// lag_piece_start so that few sequences still fill the GPU.  A later piece forms
 // its first chunk's previous range from that chunk's rows (bf16 minima and
 // maxima, the same in any order) and leaves the saved state alone; the first
 // piece, the only one that reads the state, also writes the state that the
@@ -528,7 +528,7 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
   if (SPLIT && !whole) {
     if (t_lo > 0 || !need_norm) return;
     // the state after the call's last token: its last complete chunk's range
-    // and the running one (all of these rows are the call's, lag_piece)
+    // and the running one (all of these rows are the call's, lag_piece_start)
     const int tail = (p0 + n_new) % dm.lag, tc = n_new - tail;
     uint4 pmn, pmx;
     range_of(tc - dm.lag, tc, pmn, pmx);
@@ -562,19 +562,6 @@ __device__ __forceinline__ void lag_stream(const DevState& st, const Dims& dm, c
 #else
 #define EPIKV_LAG_BOUNDS __launch_bounds__(256, EPIKV_LAG_MINB)
 #endif
-// Piece z of a call's n_new tokens starting at position p0, in pieces of
-// `piece` tokens (a multiple of lag, at least 4 * lag; 0: one piece): the
-// cuts lie at chunk boundaries, the first piece is two chunks shorter (it
-// reads up to that much at the end of the call for the state), and the rows
-// of the chunk before every cut belong to the call.
-__device__ __forceinline__ int lag_piece_start(int p0, int lag, int piece, int z) {
-  return z == 0 ? 0 : (lag - p0 % lag) % lag + z * piece - 2 * lag;
-}
-// grid.z that covers max_new tokens from any position
-static int lag_pieces(int max_new, int lag, int piece) {
-  return piece ? (max_new + 2 * lag + piece - 1) / piece : 1;
-}
-
 // SPLIT: the instance that takes calls in pieces (the other keeps the
 // registers of one piece).
 template <int LH, int KINDS, bool SPLIT>
@@ -1191,38 +1178,6 @@ cudaError_t finalize_prepare() {
   return e;
 }
 
-#ifndef EPIKV_LAG_PIECE
-#define EPIKV_LAG_PIECE 128  // shortest piece (tokens); never under 8 chunks, nor 4 in small calls
-#endif
-#ifndef EPIKV_LAG_CTAS
-#define EPIKV_LAG_CTAS 56    // CTAs per SM wanted before pieces get longer: 8 rounds of 7 resident ones
-#endif
-// Tokens per piece of the K/V scoring kernel (lag_piece_start), 0 for one
-// piece per stream.  One CTA per (layer, K|V, sequence) leaves a call of few
-// sequences at one or two CTAs per SM, each a serial chain of loads: 4
-// prompts of 4,099 to 517 tokens, 32 layers, took 695 us (1.7 TB/s), all six
-// kinds of 2 prompts of 1,500 and 1,111 tokens 502 us.  Cut into pieces:
-// 231 us (5.2 TB/s) and 125 us.  A piece re-reads the chunk before it (L2),
-// so it has at least 8 chunks; 128 against 256 tokens 125 / 139 us on the
-// second call, and 7, 14, 28, 100 CTAs per SM 274, 247, 234, 224 us on the
-// first.  A call of less than two pieces stays whole (128 tokens of 32
-// sequences fill the GPU as they are).
-static int lag_piece_tokens(const Dims& dm, int n_seq, int max_new, int num_sms) {
-  const int64_t lag = dm.lag, streams = (int64_t)2 * dm.L * n_seq;
-  // half as long where whole pieces would not even fill one round of 7 CTAs
-  // per SM: one prompt of 700 tokens 35 -> 29 us
-  const bool few = streams * max_new < (int64_t)7 * num_sms * EPIKV_LAG_PIECE;
-  const int64_t shortest = EPIKV_LAG_PIECE >> few, chunks = 8 >> few;
-  const int64_t least = (shortest > chunks * lag ? (shortest + lag - 1) / lag * lag : chunks * lag);
-  if (max_new < 2 * least) return 0;
-  const int64_t want = (int64_t)EPIKV_LAG_CTAS * num_sms;
-  const int64_t pieces = (want + streams - 1) / streams;
-  int64_t piece = (max_new + pieces - 1) / pieces;
-  piece = (piece + lag - 1) / lag * lag;
-  if (piece < least) piece = least;
-  return piece < max_new ? (int)piece : 0;
-}
-
 cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, const int32_t* seq_ids,
                                 const int32_t* cu_new, int max_new, const epikv_hidden_view* hv,
                                 const KvDev* kv, int num_sms, cudaStream_t stream, int* launches) {
@@ -1285,7 +1240,7 @@ cudaError_t launch_score_update(const DevState& st, const Dims& dm, int n_seq, c
     ++*launches;
   }
   if (dm.kinds & kKvKinds) {
-    const int piece = lag_piece_tokens(dm, n_seq, max_new, num_sms);
+    const int piece = lag_piece_tokens(dm.L, dm.lag, n_seq, max_new, num_sms);
     const dim3 grid(2 * dm.L, n_seq, lag_pieces(max_new, dm.lag, piece));
     const int threads = max(32, (dm.H * dm.d / 8 + 31) / 32 * 32);
     auto go = [&](auto kern) {

@@ -24,6 +24,17 @@ int plan_chunks(int with_late, int stash_rows, int64_t total, int G, int tails, 
                    : fill(make_chunks<false>(stash_rows, total, G, tails, stride, paged));
 }
 int plan_late_possible(int n_seq, int slots, int L, int G) { return late_possible(n_seq, slots, L, G); }
+int plan_stash_stride(int64_t total, int G, int shift, int stash_rows) {
+  return chunks_fit_stash(total, G, stash_rows) ? stash_rows : shift_stride(shift, stash_rows);
+}
+int plan_tail_start(const int32_t* kl, int first, int n_new) {
+  return tail_start([kl](int i) { return kl[i]; }, first, n_new);
+}
+int plan_lag_piece_start(int p0, int lag, int piece, int z) { return lag_piece_start(p0, lag, piece, z); }
+int plan_lag_pieces(int max_new, int lag, int piece) { return lag_pieces(max_new, lag, piece); }
+int plan_lag_piece_tokens(int L, int lag, int n_seq, int max_new, int num_sms) {
+  return lag_piece_tokens(L, lag, n_seq, max_new, num_sms);
+}
 }
 """
 _NAMES = ("kMaxStashCtas", "kStashRows", "kMaxChunks", "kPrologueRows", "kLateRows", "kLateRowsTails", "kLatePerCtaTails")
@@ -35,7 +46,7 @@ def compile_plans(out=None, defines=()):
     if cxx is None:
         raise RuntimeError("no C++ compiler found for the plans")
     consts = "".join('extern "C" int64_t const_%s() { return epikv::%s; }\n' % (n, n) for n in _NAMES)
-    cmd = [cxx, "-std=c++17", "-O1", "-Wall", "-I" + CSRC, *("-D" + d for d in defines), "-x", "c++", "-"]
+    cmd = [cxx, "-std=c++17", "-O1", "-Wall", "-Wno-unknown-pragmas", "-I" + CSRC, *("-D" + d for d in defines), "-x", "c++", "-"]
     cmd += ["-shared", "-fPIC", "-o", out] if out else ["-fsyntax-only"]
     return subprocess.run(cmd, input=_SOURCE + consts, capture_output=True, text=True)
 
@@ -50,6 +61,10 @@ class Plans:
         self._lib.plan_chunks.argtypes = [C.c_int, C.c_int, C.c_int64, C.c_int, C.c_int, C.c_int, C.c_int,
                                           C.POINTER(C.c_int64)]
         self.late_possible = self._lib.plan_late_possible
+        self.lag_piece_start = self._lib.plan_lag_piece_start
+        self.lag_pieces = self._lib.plan_lag_pieces
+        self.lag_piece_tokens = self._lib.plan_lag_piece_tokens
+        self._lib.plan_stash_stride.argtypes = [C.c_int64, C.c_int, C.c_int, C.c_int]
 
     def chunks(self, total, G, *, tails, stride, paged, stash_rows=None, late=True):
         """The first row of every chunk, and the end."""
@@ -57,6 +72,13 @@ class Plans:
         n = self._lib.plan_chunks(late, self.kStashRows if stash_rows is None else stash_rows, total, G, tails, stride,
                                   paged, out)
         return list(out[:n + 1])
+
+    def stash_stride(self, total, G, shift):
+        """Rows of a chunk's stash, 0 if the balanced split does not apply."""
+        return self._lib.plan_stash_stride(total, G, shift, self.kStashRows)
+
+    def tail_start(self, kl, first, n_new):
+        return self._lib.plan_tail_start((C.c_int32 * len(kl))(*kl), first, n_new)
 
 
 @functools.lru_cache(None)

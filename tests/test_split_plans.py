@@ -1,25 +1,15 @@
-"""The plans of the split kernels, restated and checked by brute force on the
-CPU: the chunks of long copies (one per CTA and shorter late ones, in any
-order), the head and tail split of deep cuts with its search, and the pieces
-of long K/V score updates."""
+"""The plans of the split kernels (csrc/plans.h, compiled for the host) checked
+by brute force on the CPU: the chunks of the compaction's balanced split at the
+shipped thresholds (one per CTA and, for long copies, shorter late ones, copied
+in any order), the head and tail split of deep cuts with its search, and the
+pieces of long K/V score updates.  What the kernels do with a plan (which
+sources are stashed, a batch's loads before its stores) is restated here; the
+GPU tests compare its results."""
 import random
 
 import pytest
 
-KMAX_STASH_CTAS, KMAX_CHUNKS, KCHUNKS_PAGED = 512, 1024, 768
-
-
-def chunk_starts(total, G, tails, stride, paged, stash_rows, late_rows, late_rows_tails):
-    """Chunks::start of csrc/compact.cu for every chunk, and the end."""
-    late = 0
-    if tails:
-        late = 8 * G if total >= late_rows_tails * G else 0
-    elif total >= late_rows * G:
-        late = min(min(KCHUNKS_PAGED if paged else KMAX_CHUNKS, KMAX_STASH_CTAS * stash_rows // stride) - G, 3 * G)
-    late = max(late, 0)
-    early = total - total * late // G * (20 if tails or paged else 50) // 1000 if late else total
-    n = G + late
-    return [early * c // G if c <= G else early + (total - early) * (c - G) // (n - G) for c in range(n + 1)]
+from .plans import plans
 
 
 def kept_list(rng, n, k, spread=None):
@@ -29,61 +19,57 @@ def kept_list(rng, n, k, spread=None):
     return [i for i in range(n) if i not in ev]
 
 
-def tail_start(kl, first, n_new):
-    """The eight-way search of csrc/compact.cu."""
-    lo, hi = first, n_new
-    while lo < hi:
-        step = (hi - lo + 7) // 8
-        below = sum(kl[min(lo + j * step, hi - 1)] < n_new for j in range(8))
-        if below == 0:
-            return lo
-        last = min(lo + (below - 1) * step, hi - 1)
-        if below < 8:
-            hi = min(lo + below * step, hi - 1)
-        lo = last + 1
-    return lo
-
-
-@pytest.mark.parametrize("seed", range(40))
-def test_chunks_in_any_order_leave_every_row_in_place(seed):
-    rng = random.Random(seed)
-    G, stash_rows = rng.choice([3, 8, 20]), 32
-    streams = []   # (kept, first, n_new): several streams of a few entries
-    for _ in range(rng.randint(1, 3)):
-        n = rng.randint(60, 400)
-        kl = kept_list(rng, n, n - rng.randint(1, stash_rows))
-        first = next(i for i, s in enumerate(kl) if s != i) if kl[-1] != len(kl) - 1 else len(kl)
+@pytest.mark.parametrize("late", [False, True])
+@pytest.mark.parametrize("seed", range(12))
+def test_chunks_in_any_order_leave_every_row_in_place(seed, late):
+    p, rng = plans(), random.Random(2 * seed + late)
+    G = rng.choice([1, 2, 3] if late else [3, 20, 304])
+    per_cta = rng.choice([p.kLateRows, p.kLateRows + 1, 2500] if late else [5, 100, 400, p.kLateRows - 40])
+    max_shift = rng.choice([1, 9, p.kStashRows, 300])
+    streams, n_rows = [], 0   # (kept, first, n_new, n), several streams of each entry
+    while n_rows < per_cta * G:
+        n = rng.randint(400, 1500)
+        kl = kept_list(rng, n, n - rng.randint(1, max_shift))
+        first = next((i for i, s in enumerate(kl) if s != i), len(kl))
         if first < len(kl):
             streams += [(kl, first, len(kl), n)] * rng.randint(1, 4)
+            n_rows = sum(s[2] - s[1] for s in streams)
     rows = [(s, i) for s, (kl, first, n_new, n) in enumerate(streams) for i in range(first, n_new)]
-    chunk_of = {}
-    shift = max((kl[-1] - (len(kl) - 1) for kl, *_ in streams), default=1)
-    st = chunk_starts(len(rows), G, False, shift, rng.random() < 0.5, stash_rows, 2, 2)
+    shift = max(kl[-1] - (len(kl) - 1) for kl, *_ in streams)
+    stride = p.stash_stride(len(rows), G, shift)
+    if stride == 0:
+        assert shift > p.kStashRows and -(-len(rows) // G) > p.kStashRows
+        return
+    assert stride <= p.kStashRows
+    paged = rng.random() < 0.5
+    st = p.chunks(len(rows), G, tails=False, stride=stride, paged=paged)
+    n = len(st) - 1
     assert st[0] == 0 and st[-1] == len(rows) and all(a <= b for a, b in zip(st, st[1:]))
-    assert (len(st) - 1) * shift <= KMAX_STASH_CTAS * stash_rows or len(st) - 1 == G
-    for g in range(len(st) - 1):
-        chunk_of.update((x, g) for x in rows[st[g]:st[g + 1]])
+    assert n == G if not late and len(rows) < p.kLateRows * G else n > G
+    assert n <= p.kMaxChunks and n * stride <= p.kMaxStashCtas * p.kStashRows
     cache = [list(range(n)) for *_, n in streams]
     stash = {}
-    for g in range(1, len(st) - 1):   # the sources of the chunk before, in the region from row a on
+    for g in range(1, n):   # the sources of the chunk before, in the region from row a on
         if st[g] >= len(rows):
             continue
         s, a = rows[st[g]]
         kl, first, n_new, _ = streams[s]
         if a == first:
             continue
-        start = max(first, a - (st[g] - st[g - 1]))
-        x = [i for i in range(start, a) if a <= kl[i] < n_new]
-        assert len(x) <= shift and x == list(range(x[0], x[-1] + 1)) if x else True   # a run within the stash
+        x = [i for i in range(max(first, a - (st[g] - st[g - 1])), a) if a <= kl[i] < n_new]
+        assert len(x) <= stride and (not x or x == list(range(x[0], x[-1] + 1)))   # a run within the stash
         stash[g] = {kl[i]: cache[s][kl[i]] for i in x}
-    order = list(range(len(st) - 1))
+    order = list(range(n))
     rng.shuffle(order)
     for g in order:
-        for s, i in rows[st[g]:st[g + 1]]:
+        o = st[g]
+        while o < st[g + 1]:
+            s, i = rows[o]
             kl, first, n_new, _ = streams[s]
-            end = next((e for e in range(i + 1, n_new) if chunk_of[s, e] != g), n_new)
-            stashed = end < n_new and end <= kl[i] < n_new
-            cache[s][i] = stash[g + 1][kl[i]] if stashed else cache[s][kl[i]]
+            end = min(n_new, i + st[g + 1] - o)   # the chunk's rows of this stream; another chunk's follow if end < n_new
+            for r in range(i, end):
+                cache[s][r] = stash[g + 1][kl[r]] if end < n_new and end <= kl[r] < n_new else cache[s][kl[r]]
+            o += end - i
     for (kl, first, n_new, n), c in zip(streams, cache):
         assert c[:n_new] == kl and c[n_new:] == list(range(n_new, n))
 
@@ -96,7 +82,7 @@ def test_heads_then_tails_leave_every_row_in_place(seed):
     kl = kept_list(rng, n, k, spread=rng.choice([None, max(n - k, n // 2)]))
     n_new = len(kl)
     first = next((i for i, s in enumerate(kl) if s != i), n_new)
-    cut = tail_start(kl, first, n_new)
+    cut = plans().tail_start(kl, first, n_new)
     assert cut == first + sum(s < n_new for s in kl[first:])
     cache = list(range(n))
     batch = rng.choice([1, 7, 64])
@@ -110,15 +96,11 @@ def test_heads_then_tails_leave_every_row_in_place(seed):
     assert cache[:n_new] == kl and cache[n_new:] == list(range(n_new, n))
 
 
-@pytest.mark.parametrize("seed", range(60))
-def test_pieces_cover_a_call_and_cut_at_chunks(seed):
-    rng = random.Random(2000 + seed)
-    lag = rng.choice([1, 2, 7, 16, 100])
-    piece = lag * rng.randint(4, 20)
-    p0, max_new = rng.randint(0, 5 * lag), rng.randint(1, 40 * piece // lag + 3 * piece)
-    z_n = (max_new + 2 * lag + piece - 1) // piece
-    start = [0 if z == 0 else (lag - p0 % lag) % lag + z * piece - 2 * lag for z in range(z_n + 1)]
-    for n_new in {max_new, rng.randint(0, max_new)}:
+def _check_pieces(p0, lag, piece, max_new, lengths):
+    p = plans()
+    z_n = p.lag_pieces(max_new, lag, piece)
+    start = [p.lag_piece_start(p0, lag, piece, z) for z in range(z_n + 1)]
+    for n_new in lengths:
         taken = []
         for z in range(z_n):
             lo, hi = start[z], min(n_new, start[z + 1])
@@ -131,3 +113,26 @@ def test_pieces_cover_a_call_and_cut_at_chunks(seed):
         if n_new > start[1]:   # the first piece writes the state from the call's own rows
             tail = (p0 + n_new) % lag
             assert n_new - tail - lag >= 0
+
+
+@pytest.mark.parametrize("seed", range(60))
+def test_pieces_cover_a_call_and_cut_at_chunks(seed):
+    rng = random.Random(2000 + seed)
+    lag = rng.choice([1, 2, 7, 16, 100])
+    piece = lag * rng.randint(4, 20)
+    p0, max_new = rng.randint(0, 5 * lag), rng.randint(1, 40 * piece // lag + 3 * piece)
+    _check_pieces(p0, lag, piece, max_new, {max_new, rng.randint(0, max_new)})
+
+
+@pytest.mark.parametrize("seed", range(60))
+def test_pieces_that_calls_are_cut_into(seed):
+    rng = random.Random(3000 + seed)
+    lag, L, n_seq = rng.choice([1, 3, 7, 16, 100, 5000]), rng.choice([1, 2, 32, 80]), rng.choice([1, 2, 9, 200])
+    max_new = int(2 ** rng.uniform(0, 16))
+    piece = plans().lag_piece_tokens(L, lag, n_seq, max_new, 152)
+    if piece == 0:
+        assert plans().lag_pieces(max_new, lag, piece) == 1
+        return
+    assert piece % lag == 0 and 4 * lag <= piece < max_new and max_new >= 128
+    assert plans().lag_pieces(max_new, lag, piece) <= 65535   # grid.z
+    _check_pieces(rng.randint(0, 3 * lag), lag, piece, max_new, {max_new, 1, rng.randint(0, max_new)})
