@@ -64,7 +64,8 @@ struct DevState {
   unsigned long long* lmask_new;  // [S][T] the select kernel's new masks (scratch)
   uint32_t* lkeep;         // [S][L][ceil(T/32)] bit: layer l keeps the union slot (scratch)
   int32_t* mkept;          // [S][T] the select kernel's kept slots of the largest layer (scratch)
-  uint32_t* work;          // [2] the compaction's next unit (per-layer budgets) and finished CTAs (0 between launches)
+  uint32_t* work;          // [2] the compaction's next unit or late chunk and, under per-layer budgets, its finished CTAs
+                           // (which leave both 0; under token budgets the stash kernel zeroes the first)
   char* stash;             // [kMaxStashCtas][stash_rows][H*d] bf16: compaction boundary rows, fewer per chunk for more chunks
   int32_t* stash_row0;     // [kMaxChunks] the row whose source is each stash's first row
 };
@@ -86,11 +87,33 @@ struct KvDev {
 };
 
 // Programmatic dependent launch.  The kernels of a step are launched with
-// programmatic stream serialisation (pdl_launch): each may be scheduled while
-// the kernel before it on the stream finishes, and waits in pdl_wait -- its
-// first statement -- until that kernel has completed and its writes are
-// visible; pdl_trigger lets the next kernel be scheduled once every CTA of
-// this one has started.  Launched without the attribute, both are no-ops.
+// programmatic stream serialisation (pdl_launch): each may be scheduled once
+// every CTA of the kernel before it on the stream has called pdl_trigger or
+// ended, and pdl_wait returns when that kernel has completed and its writes are
+// visible.  Launched without the attribute, both are no-ops.
+//
+// The order that this leaves.  Every kernel waits, so it completes after the
+// one before it.  A kernel may read before its wait only what the one before
+// it does not write, and only if that one triggers after its own wait: all
+// that was launched earlier has then completed.  Those that do:
+//   score_finalize_kernel  the batch and the sequences' counters (after the g
+//                          or K/V kernel)
+//   select_kernel          in a step: the batch, budgets, triggers, prefill
+//                          lengths and policies (after the score update's last
+//                          kernel)
+//   compact_kernel         the selection's results and cache rows that the
+//                          stash kernel does not move (per-layer budgets: it
+//                          also counts units, which that kernel does not)
+//   compact_consumed_kernel  the batch and the lengths (after the copy)
+//   lagkv_partial_kernel   after the g kernel: all that it reads.  It also
+//                          writes (partials and chunk ranges, of which the g
+//                          kernel knows nothing), triggers at once and waits
+//                          only before it ends.  The kernel after it is let in
+//                          once its CTAs run, so after the g kernel's wait: the
+//                          rule above holds for that one too, which then waits
+//                          for both.
+// Every other kernel waits first.  A trigger must not move ahead of a wait, nor
+// a kernel come between two of these, without a look at this list.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -44,7 +44,7 @@
 // n rows in the head.  A batch of many streams whose heads are long keeps the
 // per-stream units.  32 layers, 2 KiB rows, units (with their 512-byte to 1
 // KiB pieces) / head + tail: 65,536, 38,940 and 12,345 slots to 4,096 (3.2 GB
-// moved) 850 / 90 + 461 us; 9,000 to 3,000 461 / 52 + 97; 3 x 8,192 to 4,096
+// moved) 850 / 90 + 461 us (late chunks: 404); 9,000 to 3,000 461 / 52 + 97; 3 x 8,192 to 4,096
 // 847 / 272 + 289 (half the rows are in the heads, at 6 TB/s); 4,396 to 4,096
 // (nearly all in the head) 575 / 167 + 22.
 //

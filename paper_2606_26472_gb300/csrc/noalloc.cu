@@ -45,7 +45,7 @@ constexpr int kSeg = 8;      // tokens per segment (never crosses a chunk bounda
 constexpr int kOffs = 256;   // row offsets looked up together
 constexpr int kTile = 32;
 constexpr int kThreads = 256;
-constexpr int64_t kSms = 152;  // of a GB300
+constexpr int64_t kSms = 152;  // of a GB300, the only target (the length of pieces, never a result, depends on it)
 #ifndef EPIKV_NOALLOC_CTAS
 #define EPIKV_NOALLOC_CTAS 18   // CTAs per SM wanted before pieces get longer: three rounds of 6 resident ones
 #endif

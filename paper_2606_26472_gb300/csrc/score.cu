@@ -242,8 +242,8 @@ __device__ __forceinline__ void lag_moments(const uint4& x, const f32x2 (&a)[4],
 // block runs its own stream (K in the first half, V in the second; H*d/8 <=
 // 128), with its own shared memory.
 // KINDS: 0 = whichever K/V kinds the context computes (runtime flags); 1 =
-// the normalised kinds only; 2 = the raw kinds only; 3 = both (compile-time,
-// so a kernel instance holds only the registers its kinds need).
+// the normalised kinds only; 2 = the raw kinds only (compile-time, so a
+// kernel instance holds only the registers its kinds need).
 #ifndef EPIKV_TOKEN_OWN_OFFSET
 #define EPIKV_TOKEN_OWN_OFFSET 1  // 0: one-token calls also look the row up through shared memory
 #endif
