@@ -131,7 +131,7 @@ def ncu_traffic(kernel):
         return None
     src = os.path.join(ROOT, "paper_2606_26472_gb300", "csrc")
     h = hashlib.sha256()
-    for f in ("compact.cu", "common.cuh"):
+    for f in ("compact.cu", "common.cuh", "plans.h"):
         h.update(open(os.path.join(src, f), "rb").read())
     for line in open(path):
         parts = line.split()

@@ -74,9 +74,10 @@ using epikv::KvDev;
 // A piece first takes the minimum and maximum of the chunk before it (bf16
 // values, kept packed; exact), so pieces are independent and one sequence
 // fills the GPU.  A call on 4,001 tokens of a 32-layer cache (524 MB) takes
-// 124 us (4.2 TB/s; bound by its instructions, two passes of arithmetic per
-// row: 75 warp instructions a row, issue active 65 %), 200 tokens 19 us; one CTA per stream walking all tokens with a
-// butterfly per sum took 2,150 and 116 us.  Tokens are taken in segments of up
+// 123 us (4.3 TB/s; bound by its instructions, two passes of arithmetic per
+// row: 348 warp instructions a row, issue active 67 %), 200 tokens 19 us; one
+// CTA per stream walking all tokens with a butterfly per sum took 2,150 and
+// 116 us.  Tokens are taken in segments of up
 // to 8 inside one chunk, their rows loaded together; the variance of a
 // token's head is taken in two passes over the normalised values, four tokens
 // at a time, their sums over the head's lanes by one transposed reduction.
